@@ -301,6 +301,7 @@ struct gf_handle {
   double omega = 1.7, eps_switch = 1e-8;
   int form = GF_OR_FIRST_ORDER, reunit_interval = 20, check_interval = 1;
   int variant = GF_SWEEP_AUTO;
+  Relax relax = relax_of(1.7);  // omega as the kernels take it
   int polish = GF_POLISH_SPLIT;
   int method = GF_METHOD_OR;
   double alpha = 0.08;
@@ -437,7 +438,7 @@ SweepArgs sweep_args(gf_handle* h, int parity, bool loop, int reverse) {
   a.measure = 0;
   a.level = 1;
   a.dep = h->n_units == 1;
-  a.omega = h->omega;
+  a.omega = h->relax;
   return a;
 }
 
@@ -1362,8 +1363,9 @@ int gf_or_sweep(gf_handle* h, int parity, double omega) {
   const int st = cur_storage(h);
   for (int p = 0; p < 2; ++p) {
     if (parity != 2 && p != parity) continue;
+  const Relax relax = omega == h->omega ? h->relax : relax_of(omega);
     SweepArgs a = sweep_args(h, p, false, p);
-    a.omega = omega;
+    a.omega = relax;
     launch_sweep(st, h->nd, h->repro, h->variant, a, h->n_tiles, h->threads, h->stream);
     GF_CK_LAUNCH(h);
   }
@@ -1416,7 +1418,10 @@ int gf_fix(gf_handle* h, double eps, int maxiter, int* iters, double* F, double*
 int gf_set_omega(gf_handle* h, double omega) {
   if (!h) return GF_EINVAL;
   if (!(omega >= 1.0 && omega < 2.0)) return fail(h, GF_EINVAL, "omega must lie in [1, 2)");
-  if (omega != h->omega) drop_graphs(h);
+  if (omega != h->omega) {
+    drop_graphs(h);
+    h->relax = relax_of(omega);
+  }
   h->omega = omega;
   return GF_OK;
 }

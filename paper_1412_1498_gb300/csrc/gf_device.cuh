@@ -20,10 +20,11 @@
 // a contiguous run and every backward link U_mu(x - mu) a shifted contiguous run (mu >
 // 0) or an interleave of two neighbouring words (mu = 0): all 128-bit coalesced.
 //
-// The arithmetic helpers below spell out every complex operation in a fixed order.
-// Compiled with -fmad=false (the "reproducible" FP64 kernels) they perform exactly the
-// IEEE operations of a plain C implementation written in the same order; compiled
-// normally, nvcc contracts them into fused multiply-adds.
+// The arithmetic helpers below spell out every complex operation in a fixed order.  The
+// matrix products come in two forms: PLAIN = true sums the products as a plain C
+// implementation does and, compiled with -fmad=false (the "reproducible" FP64 kernels),
+// performs exactly its IEEE operations; PLAIN = false (every other kernel) accumulates
+// with chains of fused multiply-adds.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -161,6 +162,97 @@ template <class T>
 __device__ __forceinline__ cx<T> cscale(cx<T> a, T s) { return {a.re * s, a.im * s}; }
 template <class T>
 __device__ __forceinline__ T cnorm2(cx<T> a) { return a.re * a.re + a.im * a.im; }
+
+__device__ __forceinline__ float gf_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double gf_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// acc + x y, and acc + x conj(y), as four fused multiply-adds.  The contraction that nvcc
+// finds in cadd(acc, cmul(x, y)) is six instructions (a multiply, a fused multiply-add and
+// an add per component), and a sum that starts at zero keeps its first addition: a product
+// of 3 x 3 matrices is 108 instructions with these where it was 162.  FP64 sweeps issue
+// nothing but such chains on a pipe of two lanes per SM: 16^4 FP64-18 half-sweep 139.6 ->
+// 97.1 us; sweeps of lattices that L2 holds are bound by issue slots.  One rounding per
+// product instead of two.
+template <class T>
+__device__ __forceinline__ void cmac(cx<T>& acc, cx<T> x, cx<T> y) {
+  acc.re = gf_fma(x.re, y.re, acc.re);
+  acc.im = gf_fma(x.re, y.im, acc.im);
+  acc.re = gf_fma(-x.im, y.im, acc.re);
+  acc.im = gf_fma(x.im, y.re, acc.im);
+}
+template <class T>
+__device__ __forceinline__ void cmac_conj(cx<T>& acc, cx<T> x, cx<T> y) {
+  acc.re = gf_fma(x.re, y.re, acc.re);
+  acc.im = gf_fma(x.im, y.re, acc.im);
+  acc.re = gf_fma(x.im, y.im, acc.re);
+  acc.im = gf_fma(-x.re, y.im, acc.im);
+}
+// x y and x conj(y): a multiply and a fused multiply-add per component
+template <class T>
+__device__ __forceinline__ cx<T> cmul_fma(cx<T> x, cx<T> y) {
+  return {gf_fma(-x.im, y.im, x.re * y.re), gf_fma(x.im, y.re, x.re * y.im)};
+}
+template <class T>
+__device__ __forceinline__ cx<T> cmul_conj_fma(cx<T> x, cx<T> y) {
+  return {gf_fma(x.im, y.im, x.re * y.re), gf_fma(-x.re, y.im, x.im * y.re)};
+}
+
+// x^(-1/2) with the error of a rounding.  The hardware's FP32 reciprocal square root is off
+// by up to 2 units in the last place and not evenly to both sides; as the normalisation of
+// an SU(2) element that makes every g stretch the links it is applied to.  One Newton step
+// removes it: F of FP32 fields after 20 sweeps was off by 3e-6 to 4e-6 (32^4, 24^4), now by
+// less than 1e-7, in the same time.
+__device__ __forceinline__ double gf_rsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ float gf_rsqrt(float x) {
+  const float r = rsqrtf(x);
+  return gf_fma(0.5f * r, gf_fma(-x * r, r, 1.f), r);
+}
+
+// Exact conversions between the precisions on the integer pipe, for kernels that the FP64
+// pipe bounds: the conversion instructions run on it (2.4 a clock and SM on this GPU, as
+// slow as an FP64 addition).  They give the bits of plain casts: finite normal values and
+// zeros by shifts, and if one of a thread's values is anything else, casts.  One test for
+// all of them keeps the casts behind a branch; a conversion that is only predicated off
+// occupies the pipe all the same (32^4 FP32-12 download, which rebuilds row 2 with 24 FP64
+// instructions: 379 us with casts, 279 us with a test per value, 178 us so).
+__device__ __forceinline__ bool widens_by_shift(float x) {
+  const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+  return m - 0x00800000u < 0x7f000000u || m == 0u;
+}
+__device__ __forceinline__ double widen_shift(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+template <int N>
+__device__ __forceinline__ void widen(const cx<double> (&e)[N], cx<double>* m) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) m[k] = e[k];
+}
+template <int N>
+__device__ __forceinline__ void widen(const cx<float> (&e)[N], cx<double>* m) {
+  bool shift = true;
+#pragma unroll
+  for (int k = 0; k < N; ++k) shift = shift && widens_by_shift(e[k].re) && widens_by_shift(e[k].im);
+  if (shift) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) m[k] = {widen_shift(e[k].re), widen_shift(e[k].im)};
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) m[k] = {(double)e[k].re, (double)e[k].im};
+  }
+}
+// 2^-126 <= |x| < 2^127, or zero
+__device__ __forceinline__ bool narrows_by_shift(double x) {
+  const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return m - 0x38100000u < 0x0fd00000u || (m | (unsigned)__double2loint(x)) == 0u;
+}
+__device__ __forceinline__ float narrow_shift(double x) {  // to nearest even
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+  unsigned r = ((m - 0x38000000u) << 3) | (lo >> 29);
+  const unsigned rest = lo << 3;
+  r += rest > 0x80000000u ? 1u : (rest == 0x80000000u ? (r & 1u) : 0u);
+  return __uint_as_float((hi & 0x80000000u) | ((m | lo) == 0u ? 0u : r));
+}
 
 template <class T>
 __device__ __forceinline__ T gf_sqrt(T x);
@@ -385,18 +477,34 @@ struct Store<GF_FP64_8> {
 // ----------------------------------------------------------------------------------
 
 // row 2 of an SU(3) matrix from rows 0 and 1: conj(row0 x row1)
-template <class T>
+template <bool PLAIN = false, class T>
 __device__ __forceinline__ void third_row(const cx<T>* r, cx<T>* out) {
-  out[0] = cconj(csub(cmul(r[1], r[5]), cmul(r[2], r[4])));
-  out[1] = cconj(csub(cmul(r[2], r[3]), cmul(r[0], r[5])));
-  out[2] = cconj(csub(cmul(r[0], r[4]), cmul(r[1], r[3])));
+  if constexpr (PLAIN) {
+    out[0] = cconj(csub(cmul(r[1], r[5]), cmul(r[2], r[4])));
+    out[1] = cconj(csub(cmul(r[2], r[3]), cmul(r[0], r[5])));
+    out[2] = cconj(csub(cmul(r[0], r[4]), cmul(r[1], r[3])));
+  } else {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int i = (k + 1) % 3, j = (k + 2) % 3;  // conj(r0_i r1_j - r0_j r1_i)
+      const cx<T> a = r[i], b = r[3 + j], c = r[j], d = r[3 + i];
+      if constexpr (sizeof(T) == 8) {  // the conjugate's sign in the factors: no FP64 negation
+        out[k].re = gf_fma(c.im, d.im, gf_fma(-c.re, d.re, gf_fma(-a.im, b.im, a.re * b.re)));
+        out[k].im = gf_fma(c.im, d.re, gf_fma(c.re, d.im, gf_fma(-a.im, b.re, -a.re * b.im)));
+      } else {
+        cx<T> v = cmul_fma(a, b);
+        cmac(v, cneg(c), d);
+        out[k] = cconj(v);
+      }
+    }
+  }
 }
 
-template <class T, int NE>
+template <bool PLAIN = false, class T, int NE>
 __device__ __forceinline__ void to_full(const cx<T> (&e)[NE], cx<T> (&m)[9]) {
 #pragma unroll
   for (int k = 0; k < NE; ++k) m[k] = e[k];
-  if constexpr (NE == 6) third_row(e, m + 6);
+  if constexpr (NE == 6) third_row<PLAIN>(e, m + 6);
 }
 
 // Re Tr of a stored link
@@ -411,60 +519,94 @@ __device__ __forceinline__ T re_trace(const cx<T> (&e)[NE]) {
 }
 
 // out rows (NE/3 of them) = G * U, U given by its stored elements
-template <class T, int NE>
+template <bool PLAIN = false, class T, int NE>
 __device__ __forceinline__ void left_mul(const cx<T> (&G)[9], cx<T> (&e)[NE]) {
   cx<T> u[9];
-  to_full(e, u);
+  to_full<PLAIN>(e, u);
 #pragma unroll
   for (int i = 0; i < NE / 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      cx<T> acc = {T(0), T(0)};
+      cx<T> acc;
+      if constexpr (PLAIN) {
+        acc = {T(0), T(0)};
 #pragma unroll
-      for (int k = 0; k < 3; ++k) acc = cadd(acc, cmul(G[3 * i + k], u[3 * k + j]));
+        for (int k = 0; k < 3; ++k) acc = cadd(acc, cmul(G[3 * i + k], u[3 * k + j]));
+      } else {
+        acc = cmul_fma(G[3 * i], u[j]);
+        cmac(acc, G[3 * i + 1], u[3 + j]);
+        cmac(acc, G[3 * i + 2], u[6 + j]);
+      }
       e[3 * i + j] = acc;
     }
 }
 
 // stored rows = U * G^dagger (needs only the stored rows of U)
-template <class T, int NE>
+template <bool PLAIN = false, class T, int NE>
 __device__ __forceinline__ void right_mul_dag(cx<T> (&e)[NE], const cx<T> (&G)[9]) {
 #pragma unroll
   for (int i = 0; i < NE / 3; ++i) {
     cx<T> r0 = e[3 * i], r1 = e[3 * i + 1], r2 = e[3 * i + 2];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      cx<T> acc = {T(0), T(0)};
-      acc = cadd(acc, cmul(r0, cconj(G[3 * j + 0])));
-      acc = cadd(acc, cmul(r1, cconj(G[3 * j + 1])));
-      acc = cadd(acc, cmul(r2, cconj(G[3 * j + 2])));
+      cx<T> acc;
+      if constexpr (PLAIN) {
+        acc = {T(0), T(0)};
+        acc = cadd(acc, cmul(r0, cconj(G[3 * j + 0])));
+        acc = cadd(acc, cmul(r1, cconj(G[3 * j + 1])));
+        acc = cadd(acc, cmul(r2, cconj(G[3 * j + 2])));
+      } else {
+        acc = cmul_conj_fma(r0, G[3 * j + 0]);
+        cmac_conj(acc, r1, G[3 * j + 1]);
+        cmac_conj(acc, r2, G[3 * j + 2]);
+      }
       e[3 * i + j] = acc;
     }
   }
 }
 
+// |row|^2 of three complex numbers
+template <bool PLAIN, class T>
+__device__ __forceinline__ T row_norm2(const cx<T>* u) {
+  if constexpr (PLAIN) {
+    T n = T(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) n = n + (u[k].re * u[k].re + u[k].im * u[k].im);
+    return n;
+  } else {
+    T n = u[0].re * u[0].re;
+    n = gf_fma(u[0].im, u[0].im, n);
+#pragma unroll
+    for (int k = 1; k < 3; ++k) n = gf_fma(u[k].im, u[k].im, gf_fma(u[k].re, u[k].re, n));
+    return n;
+  }
+}
+
 // Gram-Schmidt projection to SU(3): normalise row 0, orthogonalise and normalise row 1,
 // row 2 = conj(row0 x row1) (stored only for 18-real links).
-template <class T, int NE>
+template <bool PLAIN = false, class T, int NE>
 __device__ __forceinline__ void reunit(cx<T> (&u)[NE]) {
-  T n0 = T(0);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) n0 = n0 + (u[k].re * u[k].re + u[k].im * u[k].im);
-  n0 = T(1) / gf_sqrt(n0);
+  const T n0 = PLAIN ? T(1) / gf_sqrt(row_norm2<PLAIN>(u)) : gf_rsqrt(row_norm2<PLAIN>(u));
 #pragma unroll
   for (int k = 0; k < 3; ++k) u[k] = cscale(u[k], n0);
-  cx<T> p = {T(0), T(0)};
+  if constexpr (PLAIN) {
+    cx<T> p = {T(0), T(0)};
 #pragma unroll
-  for (int k = 0; k < 3; ++k) p = cadd(p, cmul(cconj(u[k]), u[3 + k]));
+    for (int k = 0; k < 3; ++k) p = cadd(p, cmul(cconj(u[k]), u[3 + k]));
 #pragma unroll
-  for (int k = 0; k < 3; ++k) u[3 + k] = csub(u[3 + k], cmul(p, u[k]));
-  T n1 = T(0);
+    for (int k = 0; k < 3; ++k) u[3 + k] = csub(u[3 + k], cmul(p, u[k]));
+  } else {
+    cx<T> p = cmul_conj_fma(u[3], u[0]);  // conj(row0) . row1
+    cmac_conj(p, u[4], u[1]);
+    cmac_conj(p, u[5], u[2]);
+    p = cneg(p);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) n1 = n1 + (u[3 + k].re * u[3 + k].re + u[3 + k].im * u[3 + k].im);
-  n1 = T(1) / gf_sqrt(n1);
+    for (int k = 0; k < 3; ++k) cmac(u[3 + k], p, u[k]);
+  }
+  const T n1 = PLAIN ? T(1) / gf_sqrt(row_norm2<PLAIN>(u + 3)) : gf_rsqrt(row_norm2<PLAIN>(u + 3));
 #pragma unroll
   for (int k = 0; k < 3; ++k) u[3 + k] = cscale(u[3 + k], n1);
-  if constexpr (NE == 9) third_row(u, u + 6);
+  if constexpr (NE == 9) third_row<PLAIN>(u, u + 6);
 }
 
 // ----------------------------------------------------------------------------------

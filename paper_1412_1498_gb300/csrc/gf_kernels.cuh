@@ -17,19 +17,46 @@ namespace gf {
 // REPRO: IEEE divisions in the order of a plain C implementation; otherwise one
 // reciprocal square root and multiplications.
 // ----------------------------------------------------------------------------------
-template <class T>
-__device__ __forceinline__ T gf_rsqrt(T x);
-template <>
-__device__ __forceinline__ double gf_rsqrt<double>(double x) { return rsqrt(x); }
-template <>
-__device__ __forceinline__ float gf_rsqrt<float>(float x) { return rsqrtf(x); }
+// The overrelaxation parameter as the kernels take it.  To first order g^omega = 1 + omega
+// (g - 1), renormalised, is (a, b) -> mu (a + kappa, b) with kappa = (1 - omega) / omega and
+// any mu > 0.  mu is chosen (relax_of) so that q = mu kappa is a float to 1e-11: omega
+// rounded to FP32 changes the rate at which theta falls, by 2e-6 of theta after 24 sweeps.
+struct Relax {
+  double omega, kappa;
+  float mu, q;
+};
+
+inline Relax relax_of(double omega) {
+  Relax r;
+  r.omega = omega;
+  r.kappa = (1.0 - omega) / omega;
+  r.mu = 1.f;
+  r.q = (float)r.kappa;
+  if (r.kappa == 0.0) return r;
+  double best = 1.0;
+  for (int k = 0; k < 4096 && best > 1e-11; ++k) {
+    const double mu = 1.0 + k / 4096.0, q = mu * r.kappa;
+    const double e = (double)(float)q / q - 1.0, err = e < 0.0 ? -e : e;
+    if (err < best) {
+      best = err;
+      r.mu = (float)mu;
+      r.q = (float)q;
+    }
+  }
+  return r;
+}
+__device__ __forceinline__ double relax_mu(const Relax&, double) { return 1.0; }
+__device__ __forceinline__ double relax_q(const Relax& w, double) { return w.kappa; }
+__device__ __forceinline__ float relax_mu(const Relax& w, float) { return w.mu; }
+__device__ __forceinline__ float relax_q(const Relax& w, float) { return w.q; }
 
 template <class T, bool REPRO, int FORM>
-__device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j, T omega,
+__device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j, const Relax& w,
                                               cx<T>& a, cx<T>& b) {
   const cx<T> alpha = cadd(K[3 * i + i], cconj(K[3 * j + j]));
   const cx<T> beta = csub(K[3 * j + i], cconj(K[3 * i + j]));
   const T n2 = ((alpha.re * alpha.re + alpha.im * alpha.im) + beta.re * beta.re) + beta.im * beta.im;
+  const T omega = (T)w.omega;
   a = {T(1), T(0)};
   b = {T(0), T(0)};
   if constexpr (REPRO) {
@@ -38,6 +65,21 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
       a = {alpha.re / n, -alpha.im / n};
       b = {beta.re / n, -beta.im / n};
     }
+  } else if constexpr (FORM == GF_OR_FIRST_ORDER) {
+    if (n2 > T(0)) {
+      // (a first normalisation off by an ulp shifts kappa by as much, unlike the second one it
+      // leaves g unitary: the plain FP32 instruction serves)
+      T rn;
+      if constexpr (sizeof(T) == 4) rn = rsqrtf(n2) * relax_mu(w, T(0));
+      else rn = gf_rsqrt(n2);
+      const cx<T> a1 = {gf_fma(alpha.re, rn, relax_q(w, T(0))), -alpha.im * rn};
+      const cx<T> b1 = {beta.re * rn, -beta.im * rn};
+      // |a1 + ...|^2 >= mu^2 (1 - |kappa|)^2 > 0
+      const T rm = gf_rsqrt(((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im);
+      a = cscale(a1, rm);
+      b = cscale(b1, rm);
+    }
+    return;
   } else {
     if (n2 > T(0)) {
       const T rn = gf_rsqrt(n2);
@@ -49,19 +91,10 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
     // g^omega to first order: 1 + omega (g - 1), renormalised onto SU(2)
     const cx<T> a1 = {(T(1) - omega) + omega * a.re, omega * a.im};
     const cx<T> b1 = {omega * b.re, omega * b.im};
-    const T m2 = ((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im;
-    if constexpr (REPRO) {
-      const T m = gf_sqrt(m2);
-      if (m > T(0)) {
-        a = {a1.re / m, a1.im / m};
-        b = {b1.re / m, b1.im / m};
-      }
-    } else {
-      if (m2 > T(0)) {
-        const T rm = gf_rsqrt(m2);
-        a = cscale(a1, rm);
-        b = cscale(b1, rm);
-      }
+    const T m = gf_sqrt(((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im);
+    if (m > T(0)) {
+      a = {a1.re / m, a1.im / m};
+      b = {b1.re / m, b1.im / m};
     }
   } else {
     // exact power: R = cos(phi) + i sin(phi) n.sigma  ->  cos(omega phi) + i sin(omega phi) n.sigma
@@ -76,27 +109,36 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
 }
 
 // M <- R M for the subgroup element R on rows (i, j)
-template <class T>
+template <bool PLAIN, class T>
 __device__ __forceinline__ void su2_left_mul(cx<T> (&M)[9], int i, int j, cx<T> a, cx<T> b) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const cx<T> mi = M[3 * i + c], mj = M[3 * j + c];
-    M[3 * i + c] = cadd(cmul(a, mi), cmul(b, mj));
-    M[3 * j + c] = cadd(cmul(cneg(cconj(b)), mi), cmul(cconj(a), mj));
+    if constexpr (PLAIN) {
+      M[3 * i + c] = cadd(cmul(a, mi), cmul(b, mj));
+      M[3 * j + c] = cadd(cmul(cneg(cconj(b)), mi), cmul(cconj(a), mj));
+    } else {
+      cx<T> v = cmul_fma(a, mi), w = cmul_conj_fma(mj, a);
+      cmac(v, b, mj);
+      cmac_conj(w, cneg(mi), b);
+      M[3 * i + c] = v;
+      M[3 * j + c] = w;
+    }
   }
 }
 
 // G = product of the three subgroup maximisers for K (Cabibbo-Marinari order (0,1),
 // (0,2), (1,2)), K rotated after each one.
-// The first product R1 * 1 is R1 itself (x * 1 = x, x + 0 = x: the values of the plain
-// sequence).  K is left as R2 R1 K unless rotate_last asks for the third rotation too,
-// which leaves K = G K (used by the fused check, see site_check_from_GK).
+// The first product R1 * 1 is R1 itself, and outside the reproducible arithmetic the
+// second one, R2 R1, skips the products with R1's zeros and its 1 (a compiler may not: 0 x
+// is not 0 for every x).  K is left as R2 R1 K unless rotate_last asks for the third
+// rotation too, which leaves K = G K (used by the fused check, see site_check_from_GK).
 template <class T, bool REPRO, int FORM>
-__device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], T omega,
+__device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], const Relax& omega,
                                            bool rotate_last = false) {
   cx<T> a, b;
   su2_maximiser<T, REPRO, FORM>(K, 0, 1, omega, a, b);
-  su2_left_mul(K, 0, 1, a, b);
+  su2_left_mul<REPRO>(K, 0, 1, a, b);
 #pragma unroll
   for (int e = 0; e < 9; ++e) G[e] = {T(0), T(0)};
   G[0] = a;
@@ -105,23 +147,46 @@ __device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], T omega
   G[4] = cconj(a);
   G[8] = {T(1), T(0)};
   su2_maximiser<T, REPRO, FORM>(K, 0, 2, omega, a, b);
-  su2_left_mul(K, 0, 2, a, b);
-  su2_left_mul(G, 0, 2, a, b);
+  su2_left_mul<REPRO>(K, 0, 2, a, b);
+  if constexpr (REPRO) {
+    su2_left_mul<REPRO>(G, 0, 2, a, b);
+  } else {
+    // row 0 = (a G00, a G01, b), row 2 = (-conj(b) G00, -conj(b) G01, conj(a)); G12 = 0
+    const cx<T> nb = cneg(b);
+    G[6] = cmul_conj_fma(G[0], nb);
+    G[7] = cmul_conj_fma(G[1], nb);
+    G[8] = cconj(a);
+    G[0] = cmul_fma(a, G[0]);
+    G[1] = cmul_fma(a, G[1]);
+    G[2] = b;
+  }
   su2_maximiser<T, REPRO, FORM>(K, 1, 2, omega, a, b);
-  su2_left_mul(G, 1, 2, a, b);
-  if (rotate_last) su2_left_mul(K, 1, 2, a, b);
+  if constexpr (REPRO) {
+    su2_left_mul<REPRO>(G, 1, 2, a, b);
+  } else {
+    const cx<T> g22 = G[8];
+    su2_left_mul<REPRO>(G, 1, 2, a, b);  // (its third column is replaced: dead code)
+    G[5] = cmul_fma(b, g22);
+    G[8] = cmul_conj_fma(g22, a);
+  }
+  if (rotate_last) su2_left_mul<REPRO>(K, 1, 2, a, b);
 }
 
-// K += U_mu(x) + U_mu(x - mu)^dagger (in-place form of Eq. (5))
+// K += U_mu(x) + U_mu(x - mu)^dagger (in-place form of Eq. (5)); `first` direction: K =
+// that sum (x + 0 is x for every value a sum can hold here but -0, which K's users treat as 0)
 template <class T, int NE>
-__device__ __forceinline__ void add_to_K(cx<T> (&K)[9], const cx<T> (&f)[NE], const cx<T> (&b)[NE]) {
+__device__ __forceinline__ void add_to_K(cx<T> (&K)[9], const cx<T> (&f)[NE], const cx<T> (&b)[NE],
+                                         bool first = false) {
   cx<T> fu[9], bu[9];
   to_full(f, fu);
   to_full(b, bu);
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) K[3 * r + c] = cadd(K[3 * r + c], cadd(fu[3 * r + c], cconj(bu[3 * c + r])));
+    for (int c = 0; c < 3; ++c) {
+      const cx<T> s = cadd(fu[3 * r + c], cconj(bu[3 * c + r]));
+      K[3 * r + c] = first ? s : cadd(K[3 * r + c], s);
+    }
 }
 
 // A += U_nu(x - nu) - U_nu(x)  (Eq. (3), one direction)
@@ -231,7 +296,7 @@ struct SweepArgs {
   int cta_sums;            // persistent kernels, one unit: F and theta partials per CTA (indexed
                            // by blockIdx.x) instead of per tile
   int dep;                 // launch with programmatic stream serialisation (launch_dep)
-  double omega;
+  Relax omega;
 };
 
 struct MeasureArgs {
@@ -380,7 +445,6 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
     int idx_b[4];
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) idx_b[mu] = (1 - p) * lat.Vh + (int)(back_lexi(lat, s, mu) >> 1);
-    const T omega = (T)a.omega;
 
     cx<T> K[9], G[9];
 #pragma unroll
@@ -396,19 +460,19 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
         St::load(base, V, mu, idx_b[mu], b[mu]);
       }
 #pragma unroll
-      for (int mu = 0; mu < ND; ++mu) add_to_K(K, f[mu], b[mu]);
-      su3_update<T, REPRO, FORM>(K, G, omega, kCheckGK && measure_now);
+      for (int mu = 0; mu < ND; ++mu) add_to_K(K, f[mu], b[mu], !REPRO && mu == 0);
+      su3_update<T, REPRO, FORM>(K, G, a.omega, kCheckGK && measure_now);
       if (kCheckGK && measure_now) site_check_from_GK(K, fs, q);
       cx<T> A[9];
 #pragma unroll
       for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
 #pragma unroll
       for (int mu = 0; mu < 4; ++mu) {
-        left_mul(G, f[mu]);
-        right_mul_dag(b[mu], G);
+        left_mul<REPRO>(G, f[mu]);
+        right_mul_dag<REPRO>(b[mu], G);
         if (reunit_now) {
-          reunit(f[mu]);
-          reunit(b[mu]);
+          reunit<REPRO>(f[mu]);
+          reunit<REPRO>(b[mu]);
         }
         if (!kCheckGK && mu < ND && measure_now) add_to_A_F(A, fs, f[mu], b[mu]);
         St::store(base, V, mu, idx_f, f[mu]);
@@ -421,9 +485,9 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
         cx<T> f[NE], b[NE];
         St::load(base, V, mu, idx_f, f);
         St::load(base, V, mu, idx_b[mu], b);
-        add_to_K(K, f, b);
+        add_to_K(K, f, b, !REPRO && mu == 0);
       }
-      su3_update<T, REPRO, FORM>(K, G, omega, kCheckGK && measure_now);
+      su3_update<T, REPRO, FORM>(K, G, a.omega, kCheckGK && measure_now);
       if (kCheckGK && measure_now) site_check_from_GK(K, fs, q);
       cx<T> A[9];
 #pragma unroll
@@ -433,11 +497,11 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
         cx<T> f[NE], b[NE];
         St::load(base, V, mu, idx_f, f);
         St::load(base, V, mu, idx_b[mu], b);
-        left_mul(G, f);
-        right_mul_dag(b, G);
+        left_mul<REPRO>(G, f);
+        right_mul_dag<REPRO>(b, G);
         if (reunit_now) {
-          reunit(f);
-          reunit(b);
+          reunit<REPRO>(f);
+          reunit<REPRO>(b);
         }
         if (!kCheckGK && mu < ND && measure_now) add_to_A_F(A, fs, f, b);
         St::store(base, V, mu, idx_f, f);

@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
     int idx_b[4];
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) idx_b[mu] = (1 - p) * lat.Vh + (int)(back_lexi(lat, s, mu) >> 1);
-    const float omega = (float)a.omega;
+    const float omega = (float)a.omega.omega;
 
     // K = sum_{mu<nd} U_mu(x) + U_mu(x-mu)^+ with TwoSum on the hi parts
     acc2 K[18];
@@ -317,8 +317,9 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
       for (int c = 0; c < 3; ++c) {
         const cx<float> ki = {K[2 * (3 * i + c)].hi, K[2 * (3 * i + c) + 1].hi};
         const cx<float> kj = {K[2 * (3 * j + c)].hi, K[2 * (3 * j + c) + 1].hi};
-        const cx<float> di = cadd(cmul(am1, ki), cmul(bb, kj));
-        const cx<float> dj = cadd(cmul(mbc, ki), cmul(cam1, kj));
+        cx<float> di = cmul_fma(am1, ki), dj = cmul_fma(mbc, ki);
+        cmac(di, bb, kj);
+        cmac(dj, cam1, kj);
         acc_add(K[2 * (3 * i + c)], di.re, 0.f);
         acc_add(K[2 * (3 * i + c) + 1], di.im, 0.f);
         acc_add(K[2 * (3 * j + c)], dj.re, 0.f);
@@ -328,8 +329,11 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const cx<float> ei = E[3 * i + c], ej = E[3 * j + c];
-        cx<float> ni = cadd(ei, cadd(cmul(am1, ei), cmul(bb, ej)));
-        cx<float> nj = cadd(ej, cadd(cmul(mbc, ei), cmul(cam1, ej)));
+        cx<float> ni = ei, nj = ej;
+        cmac(ni, am1, ei);
+        cmac(ni, bb, ej);
+        cmac(nj, mbc, ei);
+        cmac(nj, cam1, ej);
         if (c == i) { ni = cadd(ni, am1); nj = cadd(nj, mbc); }
         if (c == j) { ni = cadd(ni, bb); nj = cadd(nj, cam1); }
         E[3 * i + c] = ni;
@@ -358,8 +362,8 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
             cx<float> x = {0.f, 0.f};
 #pragma unroll
             for (int k = 0; k < 3; ++k)
-              x = side == 0 ? cadd(x, cmul(E[3 * r + k], csf_hi(u[3 * k + c])))
-                            : cadd(x, cmul(csf_hi(u[3 * r + k]), cconj(E[3 * c + k])));
+              if (side == 0) cmac(x, E[3 * r + k], csf_hi(u[3 * k + c]));
+              else cmac_conj(x, csf_hi(u[3 * r + k]), E[3 * c + k]);
             du[3 * r + c] = x;
           }
 #pragma unroll

@@ -91,7 +91,6 @@ __global__ void __launch_bounds__(256) k_or_sweep_pipe(SweepArgs a) {
   int k = blockIdx.x;
   if (k >= a.n_tiles) return;
   const int B = blockDim.x;
-  const float omega = (float)a.omega;
   // with cta_sums each thread adds its sites' values over the CTA's tiles (compensated,
   // in a fixed order) and the CTA reduces once at the end: no barrier per tile
   const bool per_cta = measure_now && a.cta_sums;
@@ -119,9 +118,9 @@ __global__ void __launch_bounds__(256) k_or_sweep_pipe(SweepArgs a) {
           cx<float> f[6], b[6];
           pipe_read(slot, B, 3 * mu, f);
           pipe_read(slot, B, 12 + 3 * mu, b);
-          add_to_K(K, f, b);
+          add_to_K(K, f, b, mu == 0);
         }
-        su3_update<float, false, FORM>(K, G, omega, measure_now);
+        su3_update<float, false, FORM>(K, G, a.omega, measure_now);
         if (measure_now) site_check_from_GK(K, fs, q);
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
