@@ -44,7 +44,8 @@ void launch_fasd_finish(const FasdArgs& a, cudaStream_t s);
 void launch_fasd_zt(int storage, int nd, const FasdArgs& a, cudaStream_t s);
 void launch_fasd_xy_inv_g(int storage, int nd, const FasdArgs& a, cudaStream_t s);
 void launch_fasd_update(int storage, int nd, const FasdArgs& a, cudaStream_t s);
-size_t ad_partial_doubles(long long V);
+size_t ad_partial_doubles(const int* L);
+int ad_w_slices(const int* L);
 void launch_ad_forward(const AdArgs& a, cudaStream_t s);
 void launch_ad_backward(const AdArgs& a, cudaStream_t s);
 void launch_measure_fp64(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s);
@@ -126,7 +127,7 @@ int link_bytes(int storage) {
 struct Layout {
   size_t links, links64, staging, lats, lats64, tiles, unit_tiles, unit_lat, active, iters, partF,
       pthe, ptho, pending, usTo, unit_norm, usF, usT, uF, uT, lF, lT, state, kbuf, gbuf, planeF, planeT,
-      unit_planes, ad_g, ad_delta, ad_part, ad_ticket, total;
+      unit_planes, ad_g, ad_delta, ad_w, ad_part, ad_ticket, total;
   size_t staging_bytes;
   int max_tiles, n_units;
 };
@@ -204,11 +205,12 @@ bool plan(int n_lat, const int* dims, int gauge, int storage, int flags, Layout*
   if (flags & GF_FLAG_AUTOGRAD) {
     const long long V = (long long)dims[0] * dims[1] * dims[2] * dims[3];
     L->ad_g = take(9 * 16 * (size_t)V);
-    L->ad_delta = take(9 * 16 * (size_t)V);
-    L->ad_part = take(sizeof(double) * ad_partial_doubles(V));
+    L->ad_delta = take(4 * 16 * (size_t)V);
+    L->ad_w = take(4 * 9 * 16 * (size_t)(V / dims[3]) * ad_w_slices(dims));
+    L->ad_part = take(sizeof(double) * ad_partial_doubles(dims));
     L->ad_ticket = take(sizeof(unsigned int));
   } else {
-    L->ad_g = L->ad_delta = L->ad_part = L->ad_ticket = (size_t)-1;
+    L->ad_g = L->ad_delta = L->ad_w = L->ad_part = L->ad_ticket = (size_t)-1;
   }
   L->total = off;
   L->max_tiles = max_tiles;
@@ -309,7 +311,7 @@ struct gf_handle {
   char* gbuf = nullptr;
   float2 *d_planeF = nullptr, *d_planeT = nullptr;
   int* d_unit_planes = nullptr;
-  void *ad_g = nullptr, *ad_delta = nullptr;
+  void *ad_g = nullptr, *ad_delta = nullptr, *ad_w = nullptr;
   double* ad_part = nullptr;
   unsigned int* ad_ticket = nullptr;
   bool repro = false;
@@ -1194,6 +1196,7 @@ int gf_create_batch(int n_lat, const int* dims, int gauge, int storage, int flag
   if (h->flags & GF_FLAG_AUTOGRAD) {
     h->ad_g = w + L.ad_g;
     h->ad_delta = w + L.ad_delta;
+    h->ad_w = w + L.ad_w;
     h->ad_part = (double*)(w + L.ad_part);
     h->ad_ticket = (unsigned int*)(w + L.ad_ticket);
     if (cudaMemsetAsync(h->ad_ticket, 0, sizeof(unsigned int), h->stream) != cudaSuccess)
@@ -1479,6 +1482,9 @@ static int ad_args(gf_handle* h, const double* c, AdArgs* a) {
   a->lat = h->lats[0];
   a->c = c;
   a->g = (c64*)h->ad_g;
+  a->w = (c64*)h->ad_w;
+  a->w_slices = ad_w_slices(h->lats[0].L);
+  a->w_n = 2LL * h->lats[0].V3h * a->w_slices;
   a->delta = (c64*)h->ad_delta;
   a->part = h->ad_part;
   a->ticket = h->ad_ticket;

@@ -401,8 +401,12 @@ struct AdArgs {
   const char* links;   // FP64-18 storage of the lattice
   LatDev lat;
   const double* c;     // [V][8], canonical site order
-  c64* g;              // [V][9] scratch
-  c64* delta;          // [V][9] scratch
+  c64* g;              // scratch: 9 planes of V elements
+  c64* delta;          // scratch: 4 planes of V (Delta's upper elements, its diagonal)
+  c64* w;              // scratch: transformed links, 4 x 9 planes of w_n elements
+  long long w_n;       // sites of the w_slices time slices that w holds
+  int w_slices;
+  int w_t0;            // first of them
   double* part;        // [blocks][2]
   double* out;         // F, theta
   const double* upstream;  // dL/dF, dL/dtheta
