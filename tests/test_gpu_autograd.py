@@ -132,3 +132,28 @@ def test_sgd_first_step_is_naive_descent_and_50_steps_ascend(gf):
     assert np.all(np.diff(Fs) > -1e-13) and Fs[-1] > Fs[0]
     assert hist[-1][1] < hist[0][1]
     fx.close()
+
+
+@pytest.mark.parametrize("gauge", [0, 1])
+def test_slabs_equal_the_whole(gf, gauge):
+    # 32 x 32 x 64 x 256 sites are above the link buffer (8 GiB), so the passes run in slabs of
+    # time slices (226 and 30).  The field repeats an 8 x 8 x 8 x 16 one: F, theta are its, and the
+    # gradient is its over the number of copies.  Sums of equal terms in FP64: 1e-12.
+    from paper_1412_1498_gb300.autograd import functional_theta
+    small, reps = (8, 8, 8, 16), (4, 4, 8, 16)
+    big = tuple(n * r for n, r in zip(small, reps))
+    U = torch.from_numpy(fields.random_gauge_config(small, 0.5, 103)).cuda()
+    c = torch.from_numpy(np.random.default_rng(4).normal(scale=0.3, size=small[::-1] + (8,))).cuda()
+    res = []
+    for dims, r in ((small, (1, 1, 1, 1)), (big, reps)):
+        fx = gf.GaugeFixer(dims, gauge, gf.GF_FP64_18, autograd=True)
+        fx.upload(U.repeat(*r[::-1], 1, 1, 1))
+        p = c.repeat(*r[::-1], 1).reshape(-1, 8).contiguous().requires_grad_(True)
+        F, th = functional_theta(p, fx)
+        (g,) = torch.autograd.grad(0.3 * th - F, p)
+        res.append((F.item(), th.item(), g.reshape(dims[::-1] + (8,)) * float(np.prod(r))))
+        fx.close()
+        del fx, p
+    (F0, t0, g0), (F1, t1, g1) = res
+    assert abs(F1 - F0) < 1e-12 * abs(F0) + 1e-15 and abs(t1 - t0) < 1e-12 * t0
+    assert float((g1 - g0.repeat(*reps[::-1], 1)).abs().max()) < 1e-12 * float(g0.abs().max())
