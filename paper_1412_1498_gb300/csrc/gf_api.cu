@@ -301,9 +301,9 @@ struct gf_handle {
   int n_tiles = 0, n_units = 0, threads = 128;
   // settings
   double omega = 1.7, eps_switch = 1e-8;
+  Relax relax = relax_of(1.7);  // omega as the kernels take it
   int form = GF_OR_FIRST_ORDER, reunit_interval = 20, check_interval = 1;
   int variant = GF_SWEEP_AUTO;
-  Relax relax = relax_of(1.7);  // omega as the kernels take it
   int polish = GF_POLISH_SPLIT;
   int method = GF_METHOD_OR;
   double alpha = 0.08;
@@ -1308,20 +1308,19 @@ int gf_upload(gf_handle* h, int lat, const double* links, int on_device) {
   const double* mapped = on_device ? nullptr : host_mapped(links);
   if (on_device || mapped) {
     // device memory, or pinned host memory the kernel reads directly over the host link
-    launch_pack(h->storage, h->links, d, on_device ? links : mapped, 0, d.V, h->stream);
+    launch_pack(h->storage, h->links, d, on_device ? links : mapped, 0, d.V, h->d_active, h->d_iters, h->n_units,
+                h->stream);
     GF_CK_LAUNCH(h);
   } else {
     const long long per = (long long)(h->L.staging_bytes / (4 * 144));
     for (long long s0 = 0; s0 < d.V; s0 += per) {
       const long long n = std::min(per, d.V - s0);
       GF_CK(h, cudaMemcpyAsync(h->staging, links + s0 * 4 * 18, (size_t)n * 4 * 144, cudaMemcpyHostToDevice, h->stream));
-      launch_pack(h->storage, h->links, d, (const double*)h->staging, s0, n, h->stream);
+      launch_pack(h->storage, h->links, d, (const double*)h->staging, s0, n, h->d_active, h->d_iters, h->n_units,
+                  h->stream);
       GF_CK_LAUNCH(h);
     }
   }
-  launch_fill_int(h->d_active, 1, h->n_units, h->stream);
-  GF_CK_LAUNCH(h);
-  GF_CK(h, cudaMemsetAsync(h->d_iters, 0, sizeof(int) * h->n_units, h->stream));
   if (!on_device) GF_CK(h, cudaStreamSynchronize(h->stream));
   return GF_OK;
 }
@@ -1334,14 +1333,14 @@ int gf_download(gf_handle* h, int lat, double* links, int on_device) {
   const int st = cur_storage(h);
   double* mapped = on_device ? nullptr : const_cast<double*>(host_mapped(links));
   if (on_device || mapped) {
-    launch_unpack(st, cur_links(h), d, on_device ? links : mapped, 0, d.V, h->stream);
+    launch_unpack(st, cur_links(h), d, on_device ? links : mapped, 0, d.V, on_device != 0, h->stream);
     GF_CK_LAUNCH(h);
     if (mapped) GF_CK(h, cudaStreamSynchronize(h->stream));
   } else {
     const long long per = (long long)(h->L.staging_bytes / (4 * 144));
     for (long long s0 = 0; s0 < d.V; s0 += per) {
       const long long n = std::min(per, d.V - s0);
-      launch_unpack(st, cur_links(h), d, (double*)h->staging, s0, n, h->stream);
+      launch_unpack(st, cur_links(h), d, (double*)h->staging, s0, n, true, h->stream);
       GF_CK_LAUNCH(h);
       GF_CK(h, cudaMemcpyAsync(links + s0 * 4 * 18, h->staging, (size_t)n * 4 * 144, cudaMemcpyDeviceToHost, h->stream));
     }
@@ -1364,9 +1363,9 @@ int gf_or_sweep(gf_handle* h, int parity, double omega) {
   if (parity < 0 || parity > 2) return fail(h, GF_EINVAL, "parity must be 0, 1 or 2");
   if (!(omega >= 1.0 && omega < 2.0)) return fail(h, GF_EINVAL, "omega must lie in [1, 2)");
   const int st = cur_storage(h);
+  const Relax relax = omega == h->omega ? h->relax : relax_of(omega);
   for (int p = 0; p < 2; ++p) {
     if (parity != 2 && p != parity) continue;
-  const Relax relax = omega == h->omega ? h->relax : relax_of(omega);
     SweepArgs a = sweep_args(h, p, false, p);
     a.omega = relax;
     launch_sweep(st, h->nd, h->repro, h->variant, a, h->n_tiles, h->threads, h->stream);
@@ -1482,10 +1481,10 @@ static int ad_args(gf_handle* h, const double* c, AdArgs* a) {
   a->lat = h->lats[0];
   a->c = c;
   a->g = (c64*)h->ad_g;
+  a->delta = (c64*)h->ad_delta;
   a->w = (c64*)h->ad_w;
   a->w_slices = ad_w_slices(h->lats[0].L);
   a->w_n = 2LL * h->lats[0].V3h * a->w_slices;
-  a->delta = (c64*)h->ad_delta;
   a->part = h->ad_part;
   a->ticket = h->ad_ticket;
   a->nd = h->nd;

@@ -380,33 +380,47 @@ void launch_finish(const FinishArgs& a, cudaStream_t s) {
 // element kernels
 // ---------------------------------------------------------------------------------
 // Canonical <-> storage.  A block takes kPackLinks consecutive canonical links (9
-// complex128 each, site-major): the canonical side moves through shared memory with
-// consecutive threads on consecutive 16-byte words (coalesced, also when the canonical
-// buffer is pinned host memory read or written directly over the host link); each
-// thread then converts one link.
+// complex128 each, site-major), 18 KB that lie together, and moves them between the
+// canonical buffer and shared memory asynchronously: an upload by cp.async (16 bytes a
+// thread and word, also when the canonical buffer is pinned host memory read directly over
+// the host link), a download to device memory by one bulk copy (the block's words are
+// written to pinned host memory by its threads).  Each thread converts one link.  Twelve
+// blocks share an SM, so the copies of some hide behind the conversions of others.
 constexpr int kPackLinks = 128;
 
 __device__ __forceinline__ int storage_idx(const LatDev& lat, long long s) {
-  const int sl = (int)s;  // V < 2^31 (checked at creation)
-  const int x = sl % lat.L[0];
-  int r = sl / lat.L[0];
-  const int y = r % lat.L[1];
-  r /= lat.L[1];
-  const int z = r % lat.L[2];
-  const int t = r / lat.L[2];
-  return ((x + y + z + t) & 1) * lat.Vh + (sl >> 1);
+  const unsigned sl = (unsigned)s;  // V < 2^31 (checked at creation)
+  const unsigned V3 = 2u * (unsigned)lat.V3h, t = sl / V3, s3 = sl - t * V3;
+  const unsigned q1 = __umulhi(s3, lat.mx), z = __umulhi(q1, lat.my);
+  const unsigned x = s3 - q1 * (unsigned)lat.L[0], y = q1 - z * (unsigned)lat.L[1];
+  return (int)((x + y + z + t) & 1u) * lat.Vh + (int)(sl >> 1);
 }
 
+// With `active`, the units' masks and iteration counts are reset as well (an upload).
 template <int S>
 __global__ void __launch_bounds__(kPackLinks) k_pack(char* links, LatDev lat, const double2* src,
-                                                     long long s0, long long nsites) {
+                                                     long long s0, long long nsites, int* active, int* iters,
+                                                     int n_units) {
   using St = Store<S>;
   using T = typename St::T;
-  __shared__ double2 sm[kPackLinks * 9];
+  __shared__ __align__(128) double2 sm[kPackLinks * 9];
+  if (active)
+    for (int u = blockIdx.x * kPackLinks + threadIdx.x; u < n_units; u += gridDim.x * kPackLinks) {
+      active[u] = 1;
+      iters[u] = 0;
+    }
   const long long l0 = (long long)blockIdx.x * kPackLinks;  // first link of the block
   const long long nl = nsites * 4;
   const int nb = (int)(nl - l0 < kPackLinks ? nl - l0 : kPackLinks);
-  for (int w = threadIdx.x; w < nb * 9; w += kPackLinks) sm[w] = src[l0 * 9 + w];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int w = (int)threadIdx.x + k * kPackLinks;
+    if (w < nb * 9) {
+      const unsigned to = (unsigned)__cvta_generic_to_shared(sm + w);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(to), "l"(src + l0 * 9 + w) : "memory");
+    }
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
   if ((int)threadIdx.x >= nb) return;
   const long long i = l0 + threadIdx.x;
@@ -415,18 +429,18 @@ __global__ void __launch_bounds__(kPackLinks) k_pack(char* links, LatDev lat, co
   cx<T> e[St::NE];
 #pragma unroll
   for (int k = 0; k < St::NE; ++k) {
-    const double2 v = sm[threadIdx.x * 9 + k];
-    e[k] = {(T)v.x, (T)v.y};
+    const double2 w = sm[threadIdx.x * 9 + k];
+    e[k] = {(T)w.x, (T)w.y};
   }
   St::store(links + lat.off_bytes, lat.V, mu, storage_idx(lat, s), e);
 }
 
 template <int S>
 __global__ void __launch_bounds__(kPackLinks) k_unpack(const char* links, LatDev lat, double2* dst,
-                                                       long long s0, long long nsites) {
+                                                       long long s0, long long nsites, int bulk) {
   using St = Store<S>;
   using T = typename St::T;
-  __shared__ double2 sm[kPackLinks * 9];
+  __shared__ __align__(128) double2 sm[kPackLinks * 9];
   const long long l0 = (long long)blockIdx.x * kPackLinks;
   const long long nl = nsites * 4;
   const int nb = (int)(nl - l0 < kPackLinks ? nl - l0 : kPackLinks);
@@ -437,11 +451,24 @@ __global__ void __launch_bounds__(kPackLinks) k_unpack(const char* links, LatDev
     cx<T> e[St::NE];
     St::load(links + lat.off_bytes, lat.V, mu, storage_idx(lat, s), e);
     cx<double> m[9];
-#pragma unroll
-    for (int k = 0; k < St::NE; ++k) m[k] = {(double)e[k].re, (double)e[k].im};
+    widen(e, m);
     if constexpr (St::NE == 6) third_row(m, m + 6);
 #pragma unroll
     for (int k = 0; k < 9; ++k) sm[threadIdx.x * 9 + k] = make_double2(m[k].re, m[k].im);
+  }
+  if (bulk) {
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned from = (unsigned)__cvta_generic_to_shared(sm);
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst + l0 * 9), "r"(from),
+                   "r"(nb * 144)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+      // the block's shared memory has to live until it was read
+      asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+    }
+    return;
   }
   __syncthreads();
   for (int w = threadIdx.x; w < nb * 9; w += kPackLinks) dst[l0 * 9 + w] = sm[w];
@@ -470,10 +497,8 @@ __global__ void __launch_bounds__(256) k_to_fp64(const char* src, char* dst, Lat
   cx<T> e[St::NE];
   St::load(src + ls.off_bytes, ls.V, mu, idx, e);
   cx<double> m[9];
-#pragma unroll
-  for (int k = 0; k < St::NE; ++k) m[k] = {(double)e[k].re, (double)e[k].im};
-  if constexpr (St::NE == 6) third_row(m, m + 6);
-  reunit(m);
+  widen(e, m);
+  reunit(m);  // row 2 from rows 0, 1
   Store<GF_FP64_18>::store(dst + ld.off_bytes, ld.V, mu, idx, m);
 }
 
@@ -499,21 +524,21 @@ static unsigned int blocks_for(long long n, int threads) { return (unsigned int)
   }
 
 void launch_pack(int storage, char* links, const LatDev& lat, const double* src, long long s0,
-                 long long nsites, cudaStream_t s) {
+                 long long nsites, int* active, int* iters, int n_units, cudaStream_t s) {
   if (nsites <= 0) return;
   const unsigned int nb = blocks_for(nsites * 4, kPackLinks);
   const double2* p = reinterpret_cast<const double2*>(src);
-#define GF_CALL(S) k_pack<S><<<nb, kPackLinks, 0, s>>>(links, lat, p, s0, nsites)
+#define GF_CALL(S) k_pack<S><<<nb, kPackLinks, 0, s>>>(links, lat, p, s0, nsites, active, iters, n_units)
   GF_ELEM_SWITCH(storage, GF_CALL)
 #undef GF_CALL
 }
 
 void launch_unpack(int storage, const char* links, const LatDev& lat, double* dst, long long s0,
-                   long long nsites, cudaStream_t s) {
+                   long long nsites, bool device_dst, cudaStream_t s) {
   if (nsites <= 0) return;
   const unsigned int nb = blocks_for(nsites * 4, kPackLinks);
   double2* p = reinterpret_cast<double2*>(dst);
-#define GF_CALL(S) k_unpack<S><<<nb, kPackLinks, 0, s>>>(links, lat, p, s0, nsites)
+#define GF_CALL(S) k_unpack<S><<<nb, kPackLinks, 0, s>>>(links, lat, p, s0, nsites, device_dst)
   GF_ELEM_SWITCH(storage, GF_CALL)
 #undef GF_CALL
 }

@@ -598,10 +598,11 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish(FinishArgs a);
 // ----------------------------------------------------------------------------------
 // canonical (site-major complex128) -> storage, for sites [s0, s0 + nsites)
 template <int S>
-__global__ void k_pack(char* links, LatDev lat, const double2* src, long long s0, long long nsites);
+__global__ void k_pack(char* links, LatDev lat, const double2* src, long long s0, long long nsites, int* active,
+                       int* iters, int n_units);
 // storage -> canonical
 template <int S>
-__global__ void k_unpack(const char* links, LatDev lat, double2* dst, long long s0, long long nsites);
+__global__ void k_unpack(const char* links, LatDev lat, double2* dst, long long s0, long long nsites, int bulk);
 // reunitarise every link of one lattice
 template <int S>
 __global__ void k_reunit(char* links, LatDev lat);
@@ -641,9 +642,9 @@ void launch_measure(int storage, int nd, int variant, const MeasureArgs& a, int 
                     cudaStream_t s);
 void launch_finish(const FinishArgs& a, cudaStream_t s);
 void launch_pack(int storage, char* links, const LatDev& lat, const double* src, long long s0,
-                 long long nsites, cudaStream_t s);
+                 long long nsites, int* active, int* iters, int n_units, cudaStream_t s);
 void launch_unpack(int storage, const char* links, const LatDev& lat, double* dst, long long s0,
-                   long long nsites, cudaStream_t s);
+                   long long nsites, bool device_dst, cudaStream_t s);
 void launch_reunit(int storage, char* links, const LatDev& lat, cudaStream_t s);
 void launch_to_fp64(int storage, const char* src, char* dst, const LatDev& lat_src,
                     const LatDev& lat_dst, cudaStream_t s);

@@ -113,9 +113,45 @@ __device__ __forceinline__ void split_store_stream(char* base, long long V, int 
 #pragma unroll
   for (int w = 0; w < 9; ++w) __stcs(p + (long long)(w * 4 + mu) * V + idx, make_float4(u[w].re.hi, u[w].im.hi, u[w].re.lo, u[w].im.lo));
 }
-__device__ __forceinline__ csf split_of(double re, double im) {
-  const float rh = (float)re, ih = (float)im;
-  return {{rh, (float)(re - (double)rh)}, {ih, (float)(im - (double)ih)}};
+// hi = (float)x, lo = (float)(x - hi) for the nine elements of a link, by shifts where every
+// part allows it (see widen); one FP64 subtraction a real instead of four instructions of
+// that pipe
+__device__ __forceinline__ void split_of(const cx<double> (&m)[9], csf (&u)[9]) {
+  bool shift = true;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) shift = shift && narrows_by_shift(m[k].re) && narrows_by_shift(m[k].im);
+  cx<double> rest[9];
+  if (shift) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      u[k].re.hi = narrow_shift(m[k].re);
+      u[k].im.hi = narrow_shift(m[k].im);
+      rest[k] = {m[k].re - widen_shift(u[k].re.hi), m[k].im - widen_shift(u[k].im.hi)};
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      u[k].re.hi = (float)m[k].re;
+      u[k].im.hi = (float)m[k].im;
+      rest[k] = {m[k].re - (double)u[k].re.hi, m[k].im - (double)u[k].im.hi};
+    }
+  }
+  shift = true;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) shift = shift && narrows_by_shift(rest[k].re) && narrows_by_shift(rest[k].im);
+  if (shift) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      u[k].re.lo = narrow_shift(rest[k].re);
+      u[k].im.lo = narrow_shift(rest[k].im);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      u[k].re.lo = (float)rest[k].re;
+      u[k].im.lo = (float)rest[k].im;
+    }
+  }
 }
 
 // ------------------------------------------------------------------------- K(x)
@@ -447,13 +483,10 @@ __global__ void __launch_bounds__(256) k_to_split(const char* src, char* dst, La
   cx<T> e[St::NE];
   St::load(src + ls.off_bytes, ls.V, mu, idx, e);
   cx<double> m[9];
-#pragma unroll
-  for (int k = 0; k < St::NE; ++k) m[k] = {(double)e[k].re, (double)e[k].im};
-  if constexpr (St::NE == 6) third_row(m, m + 6);
-  reunit(m);
+  widen(e, m);
+  reunit(m);  // row 2 from rows 0, 1
   csf u[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) u[k] = split_of(m[k].re, m[k].im);
+  split_of(m, u);
   split_store(dst + ld.off_bytes, ld.V, mu, idx, u);
 }
 
@@ -465,10 +498,17 @@ __global__ void __launch_bounds__(256) k_split_to_fp64(char* links, LatDev lat) 
   const int mu = (int)(i / lat.V), idx = (int)(i % lat.V);
   csf u[9];
   split_load(links + lat.off_bytes, lat.V, mu, idx, u);
-  cx<double> m[9];
+  cx<float> hi[9], lo[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k)
-    m[k] = {(double)u[k].re.hi + (double)u[k].re.lo, (double)u[k].im.hi + (double)u[k].im.lo};
+  for (int k = 0; k < 9; ++k) {
+    hi[k] = {u[k].re.hi, u[k].im.hi};
+    lo[k] = {u[k].re.lo, u[k].im.lo};
+  }
+  cx<double> m[9], l[9];
+  widen(hi, m);
+  widen(lo, l);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) m[k] = cadd(m[k], l[k]);
   reunit(m);
   Store<GF_FP64_18>::store(links + lat.off_bytes, lat.V, mu, idx, m);
 }

@@ -217,3 +217,37 @@ def test_fp64_12_fix_matches_fp64_18(gf):
     assert abs(Fa - Fb) <= 1e-12 * Fa
     if a["iters"][0] == b["iters"][0]:
         assert np.abs(a["U"] - b["U"]).max() < 1e-9
+
+
+# ------------------------------------------------------------------- layout conversions
+@pytest.mark.parametrize("special", [False, True])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+def test_conversion_is_the_cast(gf, storage, special):
+    # stored elements come back as the cast to the storage's precision and back, bit for bit: by
+    # shifts where every element of a link is zero or normal, by conversions in the other
+    # links (FP32 denormals, overflow, infinity).  1600 links: a last block of 64.
+    dims = (2, 2, 2, 6 * 8 + 2)
+    rng = np.random.default_rng(7)
+    shape = dims[::-1] + (4, 3, 3)
+    U = rng.normal(size=shape) * 2.0 ** rng.integers(-100, 100, size=shape) + 1j * rng.normal(size=shape)
+    U[rng.random(shape) < 0.05] = 0.0
+    half = rng.random(shape) < 0.1                       # halfway between two floats
+    f = rng.normal(size=shape).astype(np.float32).astype(np.float64)
+    U[half] = (f * (1 + 2.0 ** -24))[half]
+    if special:
+        pick = rng.random(shape)
+        for k, v in enumerate([1e-40, -3e-45, 1e-300, 3.5e38, -np.inf, 2.0 ** -126 * (1 - 2.0 ** -30), 2.0 ** 127]):
+            U[(pick > 0.02 * k) & (pick < 0.02 * (k + 1))] = v
+    fx = gf.GaugeFixer(dims, gf.GF_LANDAU, storage)
+    rows = 3 if storage != gf.GF_FP32_12 else 2
+    with np.errstate(over="ignore", invalid="ignore"):
+        want = U if storage == gf.GF_FP64_18 else U.astype(np.complex64).astype(np.complex128)
+    for src in (U, torch.from_numpy(U).cuda(), torch.from_numpy(U).pin_memory()):
+        fx.upload(src)
+        for out in (np.empty(shape, np.complex128), torch.empty(shape, dtype=torch.complex128, device="cuda"),
+                    torch.empty(shape, dtype=torch.complex128).pin_memory()):
+            got = fx.download(out=out)
+            torch.cuda.synchronize()
+            got = got if isinstance(got, np.ndarray) else got.cpu().numpy()
+            assert np.array_equal(got[..., :rows, :].view(np.uint64), want[..., :rows, :].copy().view(np.uint64))
+    fx.close()
