@@ -296,38 +296,41 @@ __global__ void __launch_bounds__(kFasdThreads, S == GF_FP64_18 ? 2 : 4) k_fasd_
     const int p = (x + y + z + t) & 1;
     const int idx = p * lat.Vh + (int)(s.lexi >> 1);
     const char* base = a.links + lat.off_bytes;
-    cx<T> A[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
+    // Delta = A - A^+ - tr/3 (as theta_site) from its upper elements and imaginary diagonal:
+    // A itself is not needed, and of the fields transformed below only these
+    cx<T> d01, d02, d12;
+    T e0, e1, e2;
 #pragma unroll
     for (int nu = 0; nu < ND; ++nu) {
-      cx<T> f[NE], b[NE];
+      cx<T> f[NE], b[NE], fu[9], bu[9];
       St::load(base, lat.V, nu, idx, f);
       // all extents are even, so x - nu has the other parity
       St::load(base, lat.V, nu, (1 - p) * lat.Vh + (int)(back_lexi(lat, s, nu) >> 1), b);
-      fsum = fsum + re_trace(f);   // forward links only: every link once over all sites
-      add_to_A(A, f, b);
+      to_full(f, fu);
+      to_full(b, bu);
+      fsum = fsum + (fu[0].re + fu[4].re + fu[8].re);  // forward links: every link once over all sites
+      const cx<T> x01 = csub(csub(bu[1], fu[1]), cconj(csub(bu[3], fu[3])));
+      const cx<T> x02 = csub(csub(bu[2], fu[2]), cconj(csub(bu[6], fu[6])));
+      const cx<T> x12 = csub(csub(bu[5], fu[5]), cconj(csub(bu[7], fu[7])));
+      const T y0 = bu[0].im - fu[0].im, y1 = bu[4].im - fu[4].im, y2 = bu[8].im - fu[8].im;
+      d01 = nu == 0 ? x01 : cadd(d01, x01);
+      d02 = nu == 0 ? x02 : cadd(d02, x02);
+      d12 = nu == 0 ? x12 : cadd(d12, x12);
+      e0 = nu == 0 ? y0 : e0 + y0;
+      e1 = nu == 0 ? y1 : e1 + y1;
+      e2 = nu == 0 ? y2 : e2 + y2;
     }
-    // Delta = A - A^+ - tr/3 (as theta_site) and its four independent complex fields
-    cx<T> D[9];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) D[3 * r + c] = csub(A[3 * r + c], cconj(A[3 * c + r]));
-    const cx<T> sum = cadd(cadd(D[0], D[4]), D[8]);
-    const cx<T> tr = {sum.re / T(3), sum.im / T(3)};
-    D[0] = csub(D[0], tr);
-    D[4] = csub(D[4], tr);
-    D[8] = csub(D[8], tr);
-    T qq = T(0);
-#pragma unroll
-    for (int e = 0; e < 9; ++e) qq = qq + (D[e].re * D[e].re + D[e].im * D[e].im);
+    const T tr = (e0 + e1 + e2) * T(1.0 / 3.0);
+    e0 = T(2) * (e0 - tr);
+    e1 = T(2) * (e1 - tr);
+    e2 = T(2) * (e2 - tr);
+    const T qq = T(2) * (cnorm2(d01) + cnorm2(d02) + cnorm2(d12)) + (e0 * e0 + e1 * e1 + e2 * e2);
     q = q + qq;
     const int r = y * pitch + x, fs = Ly * pitch;
-    pl[r] = D[1];
-    pl[fs + r] = D[2];
-    pl[2 * fs + r] = D[5];
-    pl[3 * fs + r] = {D[0].im, D[4].im};
+    pl[r] = d01;
+    pl[fs + r] = d02;
+    pl[2 * fs + r] = d12;
+    pl[3 * fs + r] = {e0, e1};
   }
   const T v[2] = {fsum, q};
   float2 o[2];
@@ -473,8 +476,11 @@ __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async
 __device__ __forceinline__ void cp_async_wait_all_groups() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // ------------------------------------------------------------------------- C: FFT z(t), filter
-// Item: one field, one ky, KX consecutive kx (a.kx, chosen on the host so that two items'
-// columns fit in shared memory) and (Coulomb) one t.  Shared layout
+// Item: one field and KX consecutive columns (a.kx, chosen on the host so that two items'
+// columns fit in shared memory); Landau: of one ky, with all z and t; Coulomb: of the whole
+// (kx, ky) plane of one t, up to 128 of them, one z line per thread (with the columns of one
+// ky only, a 16^3 slice kept 16 of a
+// block's 128 threads busy: 16^3x32 FP64 165 -> 55 us an iteration).  Shared layout
 // col[kxl + KX z + (KX Lz + KX) tl]: the pad keeps both transform directions free of bank
 // conflicts.  Persistent blocks walk the items; with a.zt_prefetch the next item's
 // columns arrive by cp.async in a second buffer while the current one is transformed.
@@ -503,9 +509,11 @@ __global__ void __launch_bounds__(kFasdThreads, 2) k_fasd_zt(FasdArgs a) {
   const LatDev& lat = a.lat;
   const int Lx = lat.L[0], Ly = lat.L[1], Lz = lat.L[2], Lt = lat.L[3];
   const int lz = a.logL[2];
-  const int KX = a.kx, lk = __ffs(KX) - 1, nxg = Lx / KX;
+  const int KX = a.kx, lk = __ffs(KX) - 1;
   const int nt = ND == 4 ? Lt : 1;
-  const int n_items = nxg * Ly * (ND == 4 ? 4 : 4 * Lt);
+  // column groups: of one ky (Landau), of the plane (Coulomb, where ky stays 0 and kx0 counts on)
+  const int nxg = ND == 4 ? Lx / KX : Lx * Ly / KX, nky = ND == 4 ? Ly : 1;
+  const int n_items = nxg * nky * (ND == 4 ? 4 : 4 * Lt);
   const int pitch = KX * Lz + KX;  // 2 pitch = 2 KX (Lz + 1): z-line groups split the banks evenly
   const int n = nt << (lz + lk);   // elements of an item
   cx<T>* buf[2] = {reinterpret_cast<cx<T>*>(smraw), reinterpret_cast<cx<T>*>(smraw) + pitch * nt};
@@ -522,14 +530,14 @@ __global__ void __launch_bounds__(kFasdThreads, 2) k_fasd_zt(FasdArgs a) {
   auto decode = [&](int it, int& kx0, int& ky, int& f, int& t0) {
     kx0 = (it % nxg) * KX;
     const int r = it / nxg;
-    ky = r % Ly;
-    const int fz = r / Ly;
+    ky = r % nky;
+    const int fz = r / nky;
     f = ND == 4 ? fz : (fz & 3);
     t0 = ND == 4 ? 0 : (fz >> 2);
   };
   auto skip = [&](int it) {
     if (ND == 3 && a.active)
-      while (it < n_items && !a.active[(it / (nxg * Ly)) >> 2]) it += gridDim.x;
+      while (it < n_items && !a.active[(it / nxg) >> 2]) it += gridDim.x;
     return it;
   };
   int it = skip((int)blockIdx.x);
@@ -572,7 +580,7 @@ __global__ void __launch_bounds__(kFasdThreads, 2) k_fasd_zt(FasdArgs a) {
             es = pitch;
             base = s2x[kx0 + (l & mk)] + pxy + s2z[l >> lk];
           } else {  // z line kxl of the slice
-            base = s2x[kx0 + l] + pxy;
+            base = s2x[(kx0 + l) & (Lx - 1)] + s2y[(kx0 + l) >> a.logL[0]];
           }
           switch (lg) {
             case 1: zt_line<T, 1>(p, es, ph, base, s2, coef); break;
@@ -589,8 +597,9 @@ __global__ void __launch_bounds__(kFasdThreads, 2) k_fasd_zt(FasdArgs a) {
       if (ND == 4) fft_lines_reg(col, twt, Lz * KX, a.logL[3], Lz * KX, 1, 0, pitch, -1);  // along t
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int kxl = i & mk, kz = (i >> lk) & mz, kt = i >> (lk + lz);
-        T p2 = s2x[kx0 + kxl] + pxy + s2z[kz];
-        if (ND == 4) p2 += s2t[kt];
+        T p2 = s2z[kz];
+        if (ND == 4) p2 += s2x[kx0 + kxl] + pxy + s2t[kt];
+        else p2 += s2x[(kx0 + kxl) & (Lx - 1)] + s2y[(kx0 + kxl) >> a.logL[0]];
         const T fac = p2 > T(0) ? coef / p2 : T(0);
         const int c = kxl + KX * kz + pitch * kt;
         col[c] = cscale(col[c], fac);

@@ -103,7 +103,7 @@ void launch_fasd_finish(const FasdArgs& a, cudaStream_t s) { k_fasd_finish<<<a.n
 void launch_fasd_zt(int storage, int nd, const FasdArgs& a, cudaStream_t s) {
   int dev = 0;
   cudaGetDevice(&dev);
-  const int n_items = a.lat.L[0] / a.kx * a.lat.L[1] * (nd == 4 ? 4 : 4 * a.lat.L[3]);
+  const int n_items = a.lat.L[0] * a.lat.L[1] / a.kx * (nd == 4 ? 4 : 4 * a.lat.L[3]);
   int g = g_zt_grid[dev < kMaxDev ? dev : 0][storage == GF_FP64_18][nd == 4];
   if (g <= 0) g = 1;
   const unsigned int grid = (unsigned int)(g < n_items ? g : n_items);
