@@ -108,7 +108,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr size_t kStagingMax = 32u << 20;  // bytes of canonical links per host copy
-constexpr int kMinThreads = 64;
+constexpr int kMinTile = 32;
 constexpr int kGraphSweeps = 16;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -139,9 +139,9 @@ bool valid_dims(const int* d) {
   return lattice_sites_checked(d, (1LL << 31) - 1) > 0;
 }
 
-int tiles_for(const int* d, int threads) {
+int tiles_for(const int* d, int tile) {
   const long long V3h = (long long)d[0] * d[1] * d[2] / 2;
-  return (int)(d[3] * ((V3h + threads - 1) / threads));
+  return (int)(d[3] * ((V3h + tile - 1) / tile));
 }
 
 // Carve the workspace: every region 256-byte aligned.
@@ -159,7 +159,7 @@ bool plan(int n_lat, const int* dims, int gauge, int storage, int flags, Layout*
     long long V = (long long)d[0] * d[1] * d[2] * d[3];
     sites += V;
     vmax = std::max(vmax, V);
-    max_tiles += tiles_for(d, kMinThreads);
+    max_tiles += tiles_for(d, kMinTile);
     n_units += gauge == GF_LANDAU ? 1 : d[3];
   }
   L->links = take((size_t)sites * 4 * link_bytes(storage));
@@ -298,7 +298,9 @@ struct gf_handle {
   DevState* d_state = nullptr;
   // host copies
   std::vector<LatDev> lats, lats64;
-  int n_tiles = 0, n_units = 0, threads = 128;
+  int n_tiles = 0, n_units = 0;
+  int threads = 128;  // block size set by the caller
+  int tile = 128;     // sites per tile = threads of a sweep block (tile_sites_of)
   // settings
   double omega = 1.7, eps_switch = 1e-8;
   Relax relax = relax_of(1.7);  // omega as the kernels take it
@@ -378,11 +380,19 @@ char* cur_links(const gf_handle* h) { return h->cur >= 1 ? h->links64 : h->links
 LatDev* cur_lats(const gf_handle* h) { return h->cur >= 1 ? h->d_lats64 : h->d_lats; }
 const LatDev& cur_lat_host(const gf_handle* h, int l) { return h->cur >= 1 ? h->lats64[l] : h->lats[l]; }
 
-// Build the tile table for the current block size and upload it.  `keep` (nullable)
+// Sites per tile.  FP64 storages take one warp: their sweeps are bound by the FP64 pipe, so
+// what counts is that every SM gets the same number of warps (eight fit at 252 registers
+// whatever the block size).  16^4 half-sweep 97 -> 87 us against blocks of
+// 128 sites (256 blocks, two on some SMs and one on others); 8^4 about three times faster.
+// Other storages take the block size of the settings.
+int tile_sites_of(const gf_handle* h) { return is_fp64_storage(h->storage) ? kMinTile : h->threads; }
+
+// Build the tile table for the current tile size and upload it.  `keep` (nullable)
 // lists per unit whether its tiles go into the table: a mixed run drops the tiles of
 // finished units (their range becomes empty) so that the launches of its last sweeps
 // cover only the units still working.
 int build_tiles(gf_handle* h, const std::vector<int>* keep = nullptr) {
+  h->tile = tile_sites_of(h);
   std::vector<int4> tiles;
   std::vector<int> unit_tiles, unit_lat;
   for (int l = 0; l < h->n_lat; ++l) {
@@ -398,7 +408,7 @@ int build_tiles(gf_handle* h, const std::vector<int>* keep = nullptr) {
       }
       const int unit = lat.unit0 + (h->gauge == GF_COULOMB ? t : 0);
       if (keep && !(*keep)[unit]) continue;
-      for (int h3 = 0; h3 < lat.V3h; h3 += h->threads) tiles.push_back(make_int4(l, t, h3, unit));
+      for (int h3 = 0; h3 < lat.V3h; h3 += h->tile) tiles.push_back(make_int4(l, t, h3, unit));
     }
   }
   unit_tiles.push_back((int)tiles.size());
@@ -498,9 +508,9 @@ FinishArgs finish_args(gf_handle* h, int mode) {
 // F and theta of every unit and lattice, all units (mode MEASURE or RESET), async.
 int enqueue_measure_all(gf_handle* h, int mode) {
   const int st = cur_storage(h);
-  launch_measure(st, h->nd, h->variant, measure_args(h, 0, false, 0), h->n_tiles, h->threads, h->stream);
+  launch_measure(st, h->nd, h->variant, measure_args(h, 0, false, 0), h->n_tiles, h->tile, h->stream);
   GF_CK_LAUNCH(h);
-  launch_measure(st, h->nd, h->variant, measure_args(h, 1, false, 1), h->n_tiles, h->threads, h->stream);
+  launch_measure(st, h->nd, h->variant, measure_args(h, 1, false, 1), h->n_tiles, h->tile, h->stream);
   GF_CK_LAUNCH(h);
   launch_finish(finish_args(h, mode), h->stream);
   GF_CK_LAUNCH(h);
@@ -518,13 +528,13 @@ int enqueue_opening(gf_handle* h) {
   const int st = cur_storage(h);
   MeasureArgs mo = measure_args(h, 1, false, 1);
   mo.part_F = h->d_partF;
-  launch_measure(st, h->nd, h->variant, mo, h->n_tiles, h->threads, h->stream);
+  launch_measure(st, h->nd, h->variant, mo, h->n_tiles, h->tile, h->stream);
   GF_CK_LAUNCH(h);
   launch_finish(finish_args(h, FINISH_OPEN), h->stream);
   GF_CK_LAUNCH(h);
   MeasureArgs me = measure_args(h, 0, false, 0);
   me.st = h->d_state;
-  launch_measure(st, h->nd, h->variant, me, h->n_tiles, h->threads, h->stream);
+  launch_measure(st, h->nd, h->variant, me, h->n_tiles, h->tile, h->stream);
   GF_CK_LAUNCH(h);
   FinishArgs fr = finish_args(h, FINISH_RESET);
   fr.gated = 1;
@@ -549,20 +559,20 @@ int enqueue_opening(gf_handle* h) {
 int enqueue_loop_sweep(gf_handle* h, cudaStream_t s, int* pass) {
   const int st = cur_storage(h);
   launch_sweep(st, h->nd, h->repro, h->variant, sweep_args(h, 0, true, (*pass)++ & 1), h->n_tiles,
-               h->threads, s);
+               h->tile, s);
   GF_CK_LAUNCH(h);
   SweepArgs ao = sweep_args(h, 1, true, (*pass)++ & 1);
   FinishArgs fo = finish_args(h, FINISH_ODD);
   if (h->n_units == 1 && st == GF_FP32_12 && h->variant != GF_SWEEP_REGISTER) {
     ao.cta_sums = 1;
-    fo.n_odd_parts = sweep_pipe_grid(h->nd, h->threads, h->n_tiles);
+    fo.n_odd_parts = sweep_pipe_grid(h->nd, h->tile, h->n_tiles);
   }
-  launch_sweep(st, h->nd, h->repro, h->variant, ao, h->n_tiles, h->threads, s);
+  launch_sweep(st, h->nd, h->repro, h->variant, ao, h->n_tiles, h->tile, s);
   GF_CK_LAUNCH(h);
   launch_finish(fo, s);
   GF_CK_LAUNCH(h);
   if (h->n_units > 1) {
-    launch_measure(st, h->nd, h->variant, measure_args(h, 0, true, ao.reverse ^ 1), h->n_tiles, h->threads, s);
+    launch_measure(st, h->nd, h->variant, measure_args(h, 0, true, ao.reverse ^ 1), h->n_tiles, h->tile, s);
     GF_CK_LAUNCH(h);
     launch_finish(finish_args(h, FINISH_LOOP), s);
     GF_CK_LAUNCH(h);
@@ -573,7 +583,7 @@ int enqueue_loop_sweep(gf_handle* h, cudaStream_t s, int* pass) {
 // The even-site theta pass for the units an open sweep left undecided, then FINISH_LOOP
 // (their theta, masks and iteration counts; the sweep is counted and the hold released).
 int resolve_open_sweep(gf_handle* h) {
-  launch_measure(cur_storage(h), h->nd, h->variant, measure_args(h, 0, true, 0), h->n_tiles, h->threads,
+  launch_measure(cur_storage(h), h->nd, h->variant, measure_args(h, 0, true, 0), h->n_tiles, h->tile,
                  h->stream);
   GF_CK_LAUNCH(h);
   launch_finish(finish_args(h, FINISH_LOOP), h->stream);
@@ -594,7 +604,7 @@ int ensure_graphs(gf_handle* h) {
     int rc = GF_OK, pass = 0;
     for (int j = 0; j < (kGraphSweeps >> k) && rc == GF_OK; ++j) rc = enqueue_loop_sweep(h, h->cap_stream, &pass);
     if (rc == GF_OK) {
-      launch_measure(cur_storage(h), h->nd, h->variant, measure_args(h, 0, true, 0), h->n_tiles, h->threads,
+      launch_measure(cur_storage(h), h->nd, h->variant, measure_args(h, 0, true, 0), h->n_tiles, h->tile,
                      h->cap_stream);
       launch_finish(finish_args(h, FINISH_LOOP), h->cap_stream);
       if (cudaGetLastError() != cudaSuccess) rc = fail(h, GF_ECUDA, "launch in the loop capture failed");
@@ -762,7 +772,7 @@ int enqueue_mixed_sweep(gf_handle* h, cudaStream_t s, int* pass, int mask) {
     for (int L = 1; L <= 3; ++L)
       if (mask & (1 << (L - 1))) {
         launch_sweep(level_storage(h, L), h->nd, h->repro, h->variant, sweep_args_level(h, L, parity, rev),
-                     h->n_tiles, h->threads, s);
+                     h->n_tiles, h->tile, s);
         GF_CK_LAUNCH(h);
       }
   }
@@ -772,7 +782,7 @@ int enqueue_mixed_sweep(gf_handle* h, cudaStream_t s, int* pass, int mask) {
     for (int L = 1; L <= 3; ++L)
       if (mask & (1 << (L - 1))) {
         launch_measure(level_storage(h, L), h->nd, h->variant, measure_args_level(h, L, 0, rev ^ 1, true),
-                       h->n_tiles, h->threads, s);
+                       h->n_tiles, h->tile, s);
         GF_CK_LAUNCH(h);
       }
     launch_finish(finish_args(h, FINISH_LOOP), s);
@@ -786,7 +796,7 @@ int resolve_open_sweep_levels(gf_handle* h, int mask) {
   for (int L = 1; L <= 3; ++L)
     if (mask & (1 << (L - 1))) {
       launch_measure(level_storage(h, L), h->nd, h->variant, measure_args_level(h, L, 0, 0, true), h->n_tiles,
-                     h->threads, h->stream);
+                     h->tile, h->stream);
       GF_CK_LAUNCH(h);
     }
   launch_finish(finish_args(h, FINISH_LOOP), h->stream);
@@ -836,7 +846,7 @@ int enqueue_enter(gf_handle* h, const std::vector<int>& pend) {
     if (levels & (1 << (L - 1)))
       for (int parity = 0; parity < 2; ++parity) {
         launch_measure(level_storage(h, L), h->nd, h->variant, measure_args_level(h, L, parity, parity, false),
-                       h->n_tiles, h->threads, h->stream);
+                       h->n_tiles, h->tile, h->stream);
         GF_CK_LAUNCH(h);
       }
   launch_finish(finish_args(h, FINISH_ENTER), h->stream);
@@ -867,7 +877,7 @@ int run_mixed(gf_handle* h, double eps, int budget, int* sweeps_fp32, int* sweep
   std::vector<long long> unit_ntiles(nu, 0);
   for (int l = 0; l < h->n_lat; ++l) {
     const LatDev& d = h->lats[l];
-    const long long per_slice = (d.V3h + h->threads - 1) / h->threads;
+    const long long per_slice = (d.V3h + h->tile - 1) / h->tile;
     for (int k = 0; k < d.n_units; ++k) unit_ntiles[d.unit0 + k] = per_slice * (d.L[3] / d.n_units);
   }
   bool compacted = false;
@@ -1368,7 +1378,7 @@ int gf_or_sweep(gf_handle* h, int parity, double omega) {
     if (parity != 2 && p != parity) continue;
     SweepArgs a = sweep_args(h, p, false, p);
     a.omega = relax;
-    launch_sweep(st, h->nd, h->repro, h->variant, a, h->n_tiles, h->threads, h->stream);
+    launch_sweep(st, h->nd, h->repro, h->variant, a, h->n_tiles, h->tile, h->stream);
     GF_CK_LAUNCH(h);
   }
   return GF_OK;
