@@ -323,10 +323,10 @@ struct gf_handle {
   int phase_sweeps[2] = {0, 0};
   int sweeps_done = 0;  // since the last upload: the reunitarisation / check schedule
   // graphs: per buffer state (OR) one of each length 16, 8, 4, 2, 1 sweeps, one per set
-  // of precision levels of a mixed run, one for Fourier acceleration
+  // of precision levels of a mixed run, the same lengths for Fourier acceleration
   cudaGraphExec_t graph[3][5] = {};
   cudaGraphExec_t graph_mix[8] = {};
-  cudaGraphExec_t graph_fasd = nullptr;
+  cudaGraphExec_t graph_fasd[6] = {};  // 16, 8, 4, 2, 1 iterations; the measurement after the last
   // pinned host ring: slots 0 and 1 receive the result block (iteration counts, lattice
   // F and theta, loop state) behind each replay in flight, whose events follow the
   // copies; slot 2 holds the loop state uploaded at the start of a phase
@@ -367,10 +367,11 @@ void drop_graphs(gf_handle* h) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
-  if (h->graph_fasd) {
-    cudaGraphExecDestroy(h->graph_fasd);
-    h->graph_fasd = nullptr;
-  }
+  for (auto& g : h->graph_fasd)
+    if (g) {
+      cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
 }
 
 int cur_storage(const gf_handle* h) {
@@ -1030,13 +1031,18 @@ FasdArgs fasd_args(gf_handle* h, bool loop, int mode) {
   return a;
 }
 
-// One iteration: Delta + F/theta (A, B), then, while running, C, D, E (E counts it).
-int enqueue_fasd_iteration(gf_handle* h, cudaStream_t s) {
-  const FasdArgs a = fasd_args(h, true, FINISH_LOOP);
+// Delta + F/theta (A, B); while running, C, D, E (E counts the iteration).
+int enqueue_fasd_measure(gf_handle* h, const FasdArgs& a, cudaStream_t s) {
   launch_fasd_delta_xy(h->storage, h->nd, a, s);
   GF_CK_LAUNCH(h);
   launch_fasd_finish(a, s);
   GF_CK_LAUNCH(h);
+  return GF_OK;
+}
+int enqueue_fasd_iteration(gf_handle* h, cudaStream_t s) {
+  const FasdArgs a = fasd_args(h, true, FINISH_LOOP);
+  int rc = enqueue_fasd_measure(h, a, s);
+  if (rc != GF_OK) return rc;
   launch_fasd_zt(h->storage, h->nd, a, s);
   GF_CK_LAUNCH(h);
   launch_fasd_xy_inv_g(h->storage, h->nd, a, s);
@@ -1046,6 +1052,33 @@ int enqueue_fasd_iteration(gf_handle* h, cudaStream_t s) {
   return GF_OK;
 }
 
+// The graph of 16 >> k iterations (k < 5), or of the measurement that follows the last
+// iteration of the budget (k = 5), captured when it is first needed (while the replay before it
+// runs, unless it is the first): a handle used once does not pay for lengths it never replays.
+int ensure_fasd_graph(gf_handle* h, int k) {
+  if (h->graph_fasd[k]) return GF_OK;
+  GF_CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  int rc = GF_OK;
+  if (k == 5) rc = enqueue_fasd_measure(h, fasd_args(h, true, FINISH_LOOP), h->cap_stream);
+  else
+    for (int j = 0; j < (kGraphSweeps >> k) && rc == GF_OK; ++j) rc = enqueue_fasd_iteration(h, h->cap_stream);
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
+  if (rc != GF_OK) {
+    if (g) cudaGraphDestroy(g);
+    return rc;
+  }
+  if (e != cudaSuccess) return fail(h, GF_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+  e = cudaGraphInstantiate(&h->graph_fasd[k], g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) return fail(h, GF_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  return GF_OK;
+}
+
+// The loop of Algorithm 2, replayed as run_phase's is: two replays in flight, each followed by
+// a copy of the result block, the lengths chosen so that little runs past the budget (one
+// graph of 16 iterations and a second one for the final measurement left up to 31 iterations'
+// launches idle).
 int run_fasd(gf_handle* h, double eps, int budget, int* done) {
   DevState st{};
   const int offset = h->sweeps_done;
@@ -1057,30 +1090,40 @@ int run_fasd(gf_handle* h, double eps, int budget, int* done) {
   st.ticket = 0;
   st.stop = 0;
   st.eps = eps;
-  GF_CK(h, cudaMemcpyAsync(h->d_state, &st, sizeof st, cudaMemcpyHostToDevice, h->stream));
+  h->res_slot = -1;
+  std::memcpy(h->res_host + 2 * h->res_stride, &st, sizeof st);
+  GF_CK(h, cudaMemcpyAsync(h->d_state, h->res_host + 2 * h->res_stride, sizeof st, cudaMemcpyHostToDevice,
+                           h->stream));
   launch_fill_int(h->d_active, 1, h->n_units, h->stream);
   GF_CK_LAUNCH(h);
-  if (!h->graph_fasd) {
-    GF_CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = GF_OK;
-    for (int j = 0; j < kGraphSweeps && rc == GF_OK; ++j) rc = enqueue_fasd_iteration(h, h->cap_stream);
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
-    if (rc != GF_OK) {
-      if (g) cudaGraphDestroy(g);
-      return rc;
-    }
-    if (e != cudaSuccess) return fail(h, GF_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&h->graph_fasd, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(h, GF_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-  }
   int rc;
-  do {  // until every unit converged or the field after the budget has been measured
-    GF_CK(h, cudaGraphLaunch(h->graph_fasd, h->stream));
-    if ((rc = read_state(h, &st)) != GF_OK) return rc;
-  } while (st.n_active > 0 && !st.stop);
+  // planned: iterations enqueued; budget + 1 once the measurement after the last one is too
+  int planned = 0, inflight = 0, w = 0, r = 0, last = 0;
+  bool stop = false;
+  for (;;) {
+    while (!stop && inflight < 2 && planned <= budget) {
+      const int k = planned < budget ? graph_index(budget - planned) : 5;
+      if ((rc = ensure_fasd_graph(h, k)) != GF_OK) return rc;
+      GF_CK(h, cudaGraphLaunch(h->graph_fasd[k], h->stream));
+      GF_CK(h, cudaMemcpyAsync(h->res_host + w * h->res_stride, h->ws + h->L.iters, h->res_bytes,
+                               cudaMemcpyDeviceToHost, h->stream));
+      GF_CK(h, cudaEventRecord(h->st_ev[w], h->stream));
+      planned += k == 5 ? 1 : kGraphSweeps >> k;
+      w ^= 1;
+      ++inflight;
+    }
+    if (inflight == 0) break;
+    GF_CK(h, cudaEventSynchronize(h->st_ev[r]));
+    st = *res_state(h, r);
+    last = r;
+    r ^= 1;
+    --inflight;
+    if (st.n_active == 0 || st.stop) stop = true;
+  }
+  if (!stop) return fail(h, GF_ECUDA, "Fourier-accelerated loop did not end");
   *done = st.sweep - offset;
+  h->last_active = st.n_active;
+  h->res_slot = last;
   return GF_OK;
 }
 
@@ -1408,9 +1451,7 @@ int gf_fix(gf_handle* h, double eps, int maxiter, int* iters, double* F, double*
     h->sweeps_done += done;
     h->phase_sweeps[is_fp64_storage(h->storage) ? 1 : 0] = done;
     if ((rc = copy_out(h, F, theta, nullptr, nullptr, iters)) != GF_OK) return rc;
-    DevState s{};
-    if ((rc = read_state(h, &s)) != GF_OK) return rc;
-    return s.n_active > 0 ? GF_ENOTCONVERGED : GF_OK;
+    return h->last_active > 0 ? GF_ENOTCONVERGED : GF_OK;
   }
   const bool mixed = (h->flags & GF_FLAG_MIXED) && h->cur == 0;
   if (mixed) {
