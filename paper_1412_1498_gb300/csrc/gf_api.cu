@@ -18,6 +18,7 @@
 
 #include "../../include/gf.h"
 #include "gf_kernels.cuh"
+#include "gf_loop.cuh"
 
 namespace gf {
 void launch_sweep_fp64(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s);
@@ -26,6 +27,8 @@ void launch_sweep_fp32(int storage, int nd, const SweepArgs& a, int n_tiles, int
 void launch_sweep_fp32_pipe(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s);
 void launch_measure_fp32_pipe(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s);
 cudaError_t prepare_sweep_pipe();
+cudaError_t prepare_loop();
+cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t s);
 int sweep_pipe_grid(int nd, int threads, int n_tiles);
 void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s);
 void launch_measure_split(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s);
@@ -725,6 +728,83 @@ int run_phase(gf_handle* h, double eps, int budget, int* done) {
   return GF_OK;
 }
 
+// Whether a call's sweeps run in the one-kernel loop (gf_loop.cuh, which says where the line
+// lies): several units, FP32 storage with full or 12-real links, the default kernel and block
+// size, no history, and few enough sites, tiles and units.
+bool loop_kernel_serves(const gf_handle* h) {
+  if (h->cur != 0 || (h->storage != GF_FP32_12 && h->storage != GF_FP32_18)) return false;
+  if (h->variant != GF_SWEEP_AUTO || h->tile != kLoopThreads || h->hist || h->n_units == 1 || h->n_units > kLoopUnits) return false;
+  long long sites = 0;
+  for (const LatDev& lat : h->lats) sites += lat.V;
+  return sites <= kLoopSites && h->n_tiles <= 4 * (kLoopSites / 2 / kLoopThreads);
+}
+
+// run_phase with the sweeps in the one-kernel loop: the opening check, then launches of up to
+// kLoopSweeps sweeps, each followed by a copy of the result block.
+int run_phase_loop(gf_handle* h, double eps, int budget, int* done) {
+  DevState s{};
+  const int offset = h->sweeps_done;
+  s.sweep = offset;
+  s.limit = offset + budget;
+  s.check_interval = h->check_interval;
+  s.reunit_interval = h->reunit_interval;
+  s.eps = eps;
+  s.eps_mid = eps;
+  s.final_level = 1;
+  s.hist_base = h->hist_sweeps - offset;
+  h->res_slot = -1;
+  std::memcpy(h->res_host + 2 * h->res_stride, &s, sizeof s);
+  GF_CK(h, cudaMemcpyAsync(h->d_state, h->res_host + 2 * h->res_stride, sizeof s, cudaMemcpyHostToDevice,
+                           h->stream));
+  int rc = enqueue_opening(h);
+  if (rc != GF_OK) return rc;
+  LoopArgs a{};
+  a.links = h->links;
+  a.lats = h->d_lats;
+  a.tiles = h->d_tiles;
+  a.unit_tiles = h->d_unit_tiles;
+  a.unit_norm = h->d_unit_norm;
+  a.active = h->d_active;
+  a.iters = h->d_iters;
+  a.part_F = h->d_partF;
+  a.part_th_even = h->d_pthe;
+  a.part_th_odd = h->d_ptho;
+  a.verdict = h->d_pending;
+  a.unit_sumF = h->d_usF;
+  a.unit_sumTh = h->d_usT;
+  a.unit_sumTh_odd = h->d_usTo;
+  a.unit_F = h->d_uF;
+  a.unit_theta = h->d_uT;
+  a.lat_F = h->d_lF;
+  a.lat_theta = h->d_lT;
+  a.st = h->d_state;
+  a.n_tiles = h->n_tiles;
+  a.n_units = h->n_units;
+  a.n_lat = h->n_lat;
+  a.nd = h->nd;
+  a.omega = h->relax;
+  for (int before = offset - 1;;) {
+    const cudaError_t e = launch_loop(h->storage, h->nd, h->form, a, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge && before == offset - 1) {
+      cudaGetLastError();  // fewer SMs than the device has (a partitioned context): launches instead
+      return run_phase(h, eps, budget, done);
+    }
+    GF_CK(h, e);
+    GF_CK(h, cudaMemcpyAsync(h->res_host, h->ws + h->L.iters, h->res_bytes, cudaMemcpyDeviceToHost, h->stream));
+    GF_CK(h, cudaStreamSynchronize(h->stream));
+    s = *res_state(h, 0);
+    if (s.fault) return fail(h, GF_ECUDA, "sweep loop: a block gave up waiting for the others");
+    if (s.n_active == 0 || s.sweep >= s.limit) break;
+    if (s.sweep <= before) return fail(h, GF_ECUDA, "sweep loop made no progress");
+    before = s.sweep;
+    GF_CK(h, cudaMemsetAsync(&h->d_state->arrived, 0, sizeof(unsigned int), h->stream));
+  }
+  *done = s.sweep - offset;
+  h->last_active = s.n_active;
+  h->res_slot = 0;
+  return GF_OK;
+}
+
 // ---------------------------------------------------------------------------------
 // Mixed precision with a precision level per lattice.  Level 1 is the handle's FP32
 // storage, level 2 the double-float polish copy, level 3 the FP64-18 copy (levels 2 and 3
@@ -1216,6 +1296,7 @@ int gf_create_batch(int n_lat, const int* dims, int gauge, int storage, int flag
     }
   {
     cudaError_t e = prepare_sweep_pipe();
+    if (e == cudaSuccess) e = prepare_loop();
     if (e != cudaSuccess) return bail(GF_ECUDA, std::string("sweep kernel set-up: ") + cudaGetErrorString(e));
   }
   const Layout& L = h->L;
@@ -1460,7 +1541,9 @@ int gf_fix(gf_handle* h, double eps, int maxiter, int* iters, double* F, double*
     if ((rc = run_mixed(h, eps, maxiter, &h->phase_sweeps[0], &h->phase_sweeps[1], &done)) != GF_OK) return rc;
     h->sweeps_done = done;
   } else {
-    if ((rc = run_phase(h, eps, maxiter, &done)) != GF_OK) return rc;
+    // (four sweeps make up for the cooperative launch, 15 to 20 us)
+    rc = maxiter >= 4 && loop_kernel_serves(h) ? run_phase_loop(h, eps, maxiter, &done) : run_phase(h, eps, maxiter, &done);
+    if (rc != GF_OK) return rc;
     h->sweeps_done += done;
     h->phase_sweeps[h->cur == 1 || is_fp64_storage(h->storage) ? 1 : 0] = done;
   }

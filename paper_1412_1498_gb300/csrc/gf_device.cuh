@@ -85,6 +85,8 @@ struct DevState {
   double eps;           // stop threshold (of the final precision level)
   double eps_mid;       // threshold of level 1 when it is not the final level (mixed runs)
   int final_level;      // 1, or 3 in a mixed run (1 FP32 storage, 2 double-float, 3 FP64)
+  unsigned int arrived; // small handles' loop kernel: blocks that reached its barriers
+  int fault;            // and whether one gave up waiting there
 };
 
 // Stop threshold of a unit at precision level lvl (a mixed run leaves level 1 at the

@@ -547,3 +547,38 @@ def test_checkpoint_resume_is_bit_exact(gf, gauge):
     fc.fix(1e-300, 43)
     assert np.array_equal(fc.download(), whole)
     fc.close()
+
+
+# ---------------------------------------------------------------- one-kernel loop of small handles
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("gauge,dims_list,eps,interval", [
+    (1, [(2, 2, 2, 2)], 1e-300, 1),                 # two tiles of 4 sites
+    (1, [(6, 10, 8, 4)], 1e-6, 1),                  # ragged tiles; units stop one by one
+    (1, [(10, 6, 14, 4)], 1e-5, 7),                 # stops between checks
+    (1, [(4, 4, 4, 128)], 1e-5, 3),                 # most units
+    (1, [(32, 32, 16, 8)], 1e-300, 1),              # most sites: more tiles than blocks
+    (0, [(4, 6, 4, 2), (8, 4, 6, 10), (2, 4, 2, 6)], 1e-6, 1),  # a batch
+])
+@pytest.mark.parametrize("storage", [1, 2])
+def test_small_handle_loop_equals_launched_loop(gf, storage, gauge, dims_list, eps, interval, form):
+    # a block size of 64 takes the loop of separate launches: the same links and sweep counts;
+    # F and theta from other tiles, summed to 2^-44
+    Us = [fields.random_gauge_config(d, 0.4, 90 + i) for i, d in enumerate(dims_list)]
+    res = []
+    for threads in (128, 64):
+        fx = gf.GaugeFixer(dims_list, gauge, storage)
+        gf.gf_set_block_size(fx.h, threads)
+        gf.gf_set_check_interval(fx.h, interval)
+        gf.gf_set_overrelax_form(fx.h, form)
+        for i, U in enumerate(Us):
+            fx.upload(U, i)
+        a = fx.fix(eps, 45)
+        b = fx.fix(eps, 23)                         # continues the schedules
+        res.append(([fx.download(i) for i in range(len(Us))], a, b, gf.gf_get_sweeps_done(fx.h), fx.functional_theta()))
+        fx.close()
+    (ua, a0, a1, na, ma), (ub, b0, b1, nb, mb) = res
+    assert na == nb and all(np.array_equal(x, y) for x, y in zip(ua, ub))
+    for x, y in ((a0, b0), (a1, b1)):
+        assert x["rc"] == y["rc"] and np.array_equal(x["iters"], y["iters"])
+        assert np.allclose(x["F"], y["F"], rtol=1e-12, atol=1e-13) and np.allclose(x["theta"], y["theta"], rtol=1e-12)
+    assert all(np.allclose(x, y, rtol=1e-12, atol=1e-13) for x, y in zip(ma, mb))
