@@ -30,6 +30,7 @@ cudaError_t prepare_sweep_pipe();
 cudaError_t prepare_loop();
 cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t s);
 int sweep_pipe_grid(int nd, int threads, int n_tiles);
+void launch_sweep_dir(int storage, int nd, const SweepArgs& a, int n_tiles, cudaStream_t s);
 void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s);
 void launch_measure_split(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s);
 void launch_to_split(int storage, const char* src, char* dst, const LatDev& ls, const LatDev& ld,
@@ -68,16 +69,24 @@ bool is_compact_storage(int storage) {
   return storage == GF_FP64_12 || storage == GF_FP64_8 || storage == GF_FP32_8;
 }
 
+// FP32-12 goes through the pipelined kernels unless the register kernel is asked for or the
+// tiles are the one-warp ones of a small lattice.
+bool uses_pipe(int storage, int variant, int tile) {
+  return storage == GF_FP32_12 && variant != GF_SWEEP_REGISTER && tile >= 64;
+}
+
 void launch_sweep(int storage, int nd, bool repro, int variant, const SweepArgs& a, int n_tiles,
                   int threads, cudaStream_t s) {
   if (storage == kSplit18) {
     launch_sweep_split(nd, a, n_tiles, threads, s);
+  } else if (a.dir && !repro) {
+    launch_sweep_dir(storage, nd, a, n_tiles, s);
   } else if (is_compact_storage(storage)) {
     launch_sweep_compact(storage, nd, a, n_tiles, threads, s);
   } else if (storage == GF_FP64_18) {
     if (repro) launch_sweep_fp64_repro(nd, a, n_tiles, threads, s);
     else launch_sweep_fp64(nd, a, n_tiles, threads, s);
-  } else if (storage == GF_FP32_12 && variant != GF_SWEEP_REGISTER) {
+  } else if (uses_pipe(storage, variant, threads)) {
     launch_sweep_fp32_pipe(nd, a, n_tiles, threads, s);
   } else {
     launch_sweep_fp32(storage, nd, a, n_tiles, threads, s);
@@ -86,7 +95,7 @@ void launch_sweep(int storage, int nd, bool repro, int variant, const SweepArgs&
 
 void launch_measure(int storage, int nd, int variant, const MeasureArgs& a, int n_tiles,
                     int threads, cudaStream_t s) {
-  if (storage == GF_FP32_12 && variant != GF_SWEEP_REGISTER) {
+  if (uses_pipe(storage, variant, threads)) {
     launch_measure_fp32_pipe(nd, a, n_tiles, threads, s);
     return;
   }
@@ -384,12 +393,26 @@ char* cur_links(const gf_handle* h) { return h->cur >= 1 ? h->links64 : h->links
 LatDev* cur_lats(const gf_handle* h) { return h->cur >= 1 ? h->d_lats64 : h->d_lats; }
 const LatDev& cur_lat_host(const gf_handle* h, int l) { return h->cur >= 1 ? h->lats64[l] : h->lats[l]; }
 
+// Whether the handle's sweeps take the direction-per-warp kernel (gf_sweep_dir.cuh, which says
+// where the line lies).  FP32 handles with many units have their loop in one kernel instead.
+constexpr long long kDirSites = 1LL << 14;
+bool dir_kernel_serves(const gf_handle* h) {
+  long long sites = 0;
+  for (const LatDev& lat : h->lats) sites += lat.V;
+  if (sites > kDirSites) return false;
+  if (h->storage == GF_FP64_18) return true;
+  return h->n_units == 1 && (h->storage == GF_FP32_18 || (h->storage == GF_FP32_12 && h->variant == GF_SWEEP_AUTO));
+}
+
 // Sites per tile.  FP64 storages take one warp: their sweeps are bound by the FP64 pipe, so
 // what counts is that every SM gets the same number of warps (eight fit at 252 registers
 // whatever the block size).  16^4 half-sweep 97 -> 87 us against blocks of
 // 128 sites (256 blocks, two on some SMs and one on others); 8^4 about three times faster.
-// Other storages take the block size of the settings.
-int tile_sites_of(const gf_handle* h) { return is_fp64_storage(h->storage) ? kMinTile : h->threads; }
+// So do the lattices of the direction-per-warp kernel, whose blocks work on 32 sites.
+// Other handles take the block size of the settings.
+int tile_sites_of(const gf_handle* h) {
+  return is_fp64_storage(h->storage) || dir_kernel_serves(h) ? kMinTile : h->threads;
+}
 
 // Build the tile table for the current tile size and upload it.  `keep` (nullable)
 // lists per unit whether its tiles go into the table: a mixed run drops the tiles of
@@ -454,6 +477,7 @@ SweepArgs sweep_args(gf_handle* h, int parity, bool loop, int reverse) {
   a.measure = 0;
   a.level = 1;
   a.dep = h->n_units == 1;
+  a.dir = h->cur == 0 && dir_kernel_serves(h);
   a.omega = h->relax;
   return a;
 }
@@ -567,7 +591,7 @@ int enqueue_loop_sweep(gf_handle* h, cudaStream_t s, int* pass) {
   GF_CK_LAUNCH(h);
   SweepArgs ao = sweep_args(h, 1, true, (*pass)++ & 1);
   FinishArgs fo = finish_args(h, FINISH_ODD);
-  if (h->n_units == 1 && st == GF_FP32_12 && h->variant != GF_SWEEP_REGISTER) {
+  if (h->n_units == 1 && uses_pipe(st, h->variant, h->tile)) {
     ao.cta_sums = 1;
     fo.n_odd_parts = sweep_pipe_grid(h->nd, h->tile, h->n_tiles);
   }
@@ -827,6 +851,7 @@ SweepArgs sweep_args_level(gf_handle* h, int L, int parity, int reverse) {
   a.links = level_links(h, L);
   a.lats = level_lats(h, L);
   a.level = L;
+  a.dir = L != 2 && dir_kernel_serves(h);
   return a;
 }
 
@@ -1601,7 +1626,7 @@ int gf_set_reproducible(gf_handle* h, int on) {
 int gf_set_block_size(gf_handle* h, int threads) {
   if (!h) return GF_EINVAL;
   if (threads != 64 && threads != 128 && threads != 256) return fail(h, GF_EINVAL, "block size must be 64, 128 or 256");
-  if (threads == h->threads) return GF_OK;
+  if (threads == h->threads && tile_sites_of(h) == h->tile) return GF_OK;
   h->threads = threads;
   return build_tiles(h);
 }
@@ -1700,8 +1725,10 @@ int gf_set_sweep_variant(gf_handle* h, int variant) {
     return fail(h, GF_EINVAL, "unknown sweep variant");
   if (variant == GF_SWEEP_PIPELINED && h->storage != GF_FP32_12)
     return fail(h, GF_EINVAL, "the pipelined sweep exists for GF_FP32_12 storage only");
-  if (variant != h->variant) drop_graphs(h);
+  if (variant == h->variant) return GF_OK;
   h->variant = variant;
+  if (tile_sites_of(h) != h->tile) return build_tiles(h);  // drops the graphs
+  drop_graphs(h);
   return GF_OK;
 }
 
@@ -1717,6 +1744,8 @@ int gf_autotune(gf_handle* h, int* threads_out, int* variant_out) {
     cands.push_back({t, GF_SWEEP_REGISTER});
     if (st == GF_FP32_12) cands.push_back({t, GF_SWEEP_PIPELINED});
   }
+  // what AUTO takes on a small lattice; reported as PIPELINED, AUTO's meaning
+  if (st == GF_FP32_12 && h->tile == kMinTile) cands.push_back({128, GF_SWEEP_AUTO});
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
@@ -1752,7 +1781,7 @@ int gf_autotune(gf_handle* h, int* threads_out, int* variant_out) {
   drop_graphs(h);
   if ((rc = gf_set_block_size(h, bt)) != GF_OK) return rc;
   if (threads_out) *threads_out = bt;
-  if (variant_out) *variant_out = bv;
+  if (variant_out) *variant_out = bv == GF_SWEEP_AUTO && h->storage == GF_FP32_12 ? GF_SWEEP_PIPELINED : bv;
   return GF_OK;
 }
 

@@ -296,6 +296,7 @@ struct SweepArgs {
   int cta_sums;            // persistent kernels, one unit: F and theta partials per CTA (indexed
                            // by blockIdx.x) instead of per tile
   int dep;                 // launch with programmatic stream serialisation (launch_dep)
+  int dir;                 // the direction-per-warp kernel (small lattices)
   Relax omega;
 };
 

@@ -582,3 +582,29 @@ def test_small_handle_loop_equals_launched_loop(gf, storage, gauge, dims_list, e
         assert x["rc"] == y["rc"] and np.array_equal(x["iters"], y["iters"])
         assert np.allclose(x["F"], y["F"], rtol=1e-12, atol=1e-13) and np.allclose(x["theta"], y["theta"], rtol=1e-12)
     assert all(np.allclose(x, y, rtol=1e-12, atol=1e-13) for x, y in zip(ma, mb))
+
+
+# ---------------------------------------------------------------- direction-per-warp sweep of small lattices
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("gauge,dims", [(0, (2, 2, 2, 2)), (0, (8, 8, 8, 8)), (0, (10, 6, 14, 4)), (0, (8, 16, 16, 8)),
+                                        (1, (2, 2, 2, 4)), (1, (6, 10, 8, 4))])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+def test_small_lattice_equals_batch_member(gf, storage, gauge, dims, form):
+    # in a batch with a lattice of 2^14 sites the small one goes through the kernels of larger
+    # handles: the same links and sweep counts; F and theta from other tiles, summed to 2^-44
+    U, filler = fields.random_gauge_config(dims, 0.4, 95), fields.random_gauge_config((16, 16, 16, 4), 0.4, 96)
+    res = []
+    for lats in ([dims], [dims, (16, 16, 16, 4)]):
+        fx = gf.GaugeFixer(lats, gauge, storage)
+        gf.gf_set_overrelax_form(fx.h, form)
+        n = 1 if gauge == 0 else dims[3]
+        fx.upload(U, 0)
+        if len(lats) > 1:
+            fx.upload(filler, 1)
+        out = fx.fix(1e-6, 43)
+        fx.or_sweep(2, 1.3)
+        res.append((fx.download(0), out["iters"][:n], out["F"][0], out["theta"][0]))
+        fx.close()
+    (ua, ia, Fa, ta), (ub, ib, Fb, tb) = res
+    assert np.array_equal(ua, ub) and np.array_equal(ia, ib)
+    assert abs(Fa - Fb) < 1e-12 and abs(ta - tb) < 1e-12 * max(ta, 1e-3)
