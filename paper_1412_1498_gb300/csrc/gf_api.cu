@@ -207,7 +207,7 @@ bool plan(int n_lat, const int* dims, int gauge, int storage, int flags, Layout*
     const size_t c = storage == GF_FP64_18 ? 16 : 8;
     const long long V = (long long)d[0] * d[1] * d[2] * d[3];
     L->kbuf = take(4 * (size_t)V * c);
-    L->gbuf = take(6 * (size_t)V * c);
+    L->gbuf = take((storage == GF_FP64_18 ? 9 : 6) * (size_t)V * c);
     L->planeF = take(sizeof(float2) * d[2] * d[3]);
     L->planeT = take(sizeof(float2) * d[2] * d[3]);
     L->unit_planes = take(sizeof(int) * (n_units + 1));
@@ -405,7 +405,7 @@ bool dir_kernel_serves(const gf_handle* h) {
 }
 
 // Sites per tile.  FP64 storages take one warp: their sweeps are bound by the FP64 pipe, so
-// what counts is that every SM gets the same number of warps (eight fit at 252 registers
+// what counts is that every SM gets the same number of warps (some ten fit
 // whatever the block size).  16^4 half-sweep 97 -> 87 us against blocks of
 // 128 sites (256 blocks, two on some SMs and one on others); 8^4 about three times faster.
 // So do the lattices of the direction-per-warp kernel, whose blocks work on 32 sites.

@@ -8,7 +8,7 @@
 //                        (alpha/2) p^2_max / p^2 / N (k = 0 mode set to 0), inverse FFT;
 //   D  k_fasd_xy_inv_g   per (z,t) plane: inverse FFT along y, x, then
 //                        g(x) = reunit(1 + Delta~(x)) (first-order exponential, Sec. 1),
-//                        rows 0 and 1 stored in lexicographic site order;
+//                        stored in lexicographic site order (FP32: rows 0 and 1);
 //   E  k_fasd_update     per site, in lexicographic order: U_mu(x) <- g(x) U_mu(x)
 //                        g(x+mu)^+ for every mu (the g of a block's forward neighbours lie
 //                        in its own and the next planes, just written: L2 hits); its last
@@ -119,7 +119,10 @@ __device__ __forceinline__ void dif_reg(cx<T> (&v)[1 << LOGL], int sign) {
         const cx<T> a = v[s + j], b = v[s + j + span];
         v[s + j] = cadd(a, b);
         cx<T> e = csub(a, b);
-        if (j != 0) e = cmul(e, twiddle<T, L>(j * (L / (2 * span)), sign));  // exp(-2 pi i j / (2 span))
+        // exp(-2 pi i j / (2 span)); -i is written out, a product with its 0 would be computed
+        // (0 x is not 0 for every x): 60 of a 32-point transform's 516 operations
+        if (2 * j == span) e = sign > 0 ? cx<T>{-e.im, e.re} : cx<T>{e.im, -e.re};
+        else if (j != 0) e = cmul(e, twiddle<T, L>(j * (L / (2 * span)), sign));
         v[s + j + span] = e;
       }
     }
@@ -231,8 +234,9 @@ __device__ __forceinline__ void g_from_delta(cx<T> d01, cx<T> d02, cx<T> d12, cx
   reunit(g);
 }
 
-// g rows 0, 1 in the links' precision, site `at` (lexicographic): FP32 as 3 float4
-// words, FP64 as 6 double2 words, each word a plane of V entries
+// g in the links' precision, site `at` (lexicographic): FP32 rows 0, 1 as 3 float4 words, FP64 all
+// rows as 9 double2 words (rebuilding row 2 took 10% of the update's FP64 instructions), each
+// word a plane of V entries
 template <class T>
 __device__ __forceinline__ void g_store(char* gbuf, long long V, long long at, const cx<T> (&g)[9]) {
   if constexpr (sizeof(T) == 4) {
@@ -242,10 +246,10 @@ __device__ __forceinline__ void g_store(char* gbuf, long long V, long long at, c
   } else {
     double2* p = reinterpret_cast<double2*>(gbuf);
 #pragma unroll
-    for (int w = 0; w < 6; ++w) p[w * V + at] = make_double2(g[w].re, g[w].im);
+    for (int w = 0; w < 9; ++w) p[w * V + at] = make_double2(g[w].re, g[w].im);
   }
 }
-// rows 0, 1 (and row 2 = conj(row0 x row1) when full)
+// rows 0, 1 (FP32: row 2 = conj(row0 x row1) when full)
 template <class T, bool FULL>
 __device__ __forceinline__ void g_load(const char* gbuf, long long V, long long at, cx<T> (&g)[9]) {
   if constexpr (sizeof(T) == 4) {
@@ -258,16 +262,16 @@ __device__ __forceinline__ void g_load(const char* gbuf, long long V, long long 
       g[2 * w + 1].re = v.z;
       g[2 * w + 1].im = v.w;
     }
+    if constexpr (FULL) third_row(g, g + 6);
   } else {
     const double2* p = reinterpret_cast<const double2*>(gbuf);
 #pragma unroll
-    for (int w = 0; w < 6; ++w) {
+    for (int w = 0; w < 9; ++w) {
       const double2 v = p[w * V + at];
       g[w].re = v.x;
       g[w].im = v.y;
     }
   }
-  if constexpr (FULL) third_row(g, g + 6);
 }
 
 // ------------------------------------------------------------------------- A: Delta + FFT xy
@@ -296,10 +300,7 @@ __global__ void __launch_bounds__(kFasdThreads, S == GF_FP64_18 ? 2 : 4) k_fasd_
     const int p = (x + y + z + t) & 1;
     const int idx = p * lat.Vh + (int)(s.lexi >> 1);
     const char* base = a.links + lat.off_bytes;
-    // Delta = A - A^+ - tr/3 (as theta_site) from its upper elements and imaginary diagonal:
-    // A itself is not needed, and of the fields transformed below only these
-    cx<T> d01, d02, d12;
-    T e0, e1, e2;
+    AntiHermSum<T> D;  // Delta: the fields transformed below are its upper elements and diagonal
 #pragma unroll
     for (int nu = 0; nu < ND; ++nu) {
       cx<T> f[NE], b[NE], fu[9], bu[9];
@@ -309,28 +310,15 @@ __global__ void __launch_bounds__(kFasdThreads, S == GF_FP64_18 ? 2 : 4) k_fasd_
       to_full(f, fu);
       to_full(b, bu);
       fsum = fsum + (fu[0].re + fu[4].re + fu[8].re);  // forward links: every link once over all sites
-      const cx<T> x01 = csub(csub(bu[1], fu[1]), cconj(csub(bu[3], fu[3])));
-      const cx<T> x02 = csub(csub(bu[2], fu[2]), cconj(csub(bu[6], fu[6])));
-      const cx<T> x12 = csub(csub(bu[5], fu[5]), cconj(csub(bu[7], fu[7])));
-      const T y0 = bu[0].im - fu[0].im, y1 = bu[4].im - fu[4].im, y2 = bu[8].im - fu[8].im;
-      d01 = nu == 0 ? x01 : cadd(d01, x01);
-      d02 = nu == 0 ? x02 : cadd(d02, x02);
-      d12 = nu == 0 ? x12 : cadd(d12, x12);
-      e0 = nu == 0 ? y0 : e0 + y0;
-      e1 = nu == 0 ? y1 : e1 + y1;
-      e2 = nu == 0 ? y2 : e2 + y2;
+      D.add(fu, bu, nu == 0);
     }
-    const T tr = (e0 + e1 + e2) * T(1.0 / 3.0);
-    e0 = T(2) * (e0 - tr);
-    e1 = T(2) * (e1 - tr);
-    e2 = T(2) * (e2 - tr);
-    const T qq = T(2) * (cnorm2(d01) + cnorm2(d02) + cnorm2(d12)) + (e0 * e0 + e1 * e1 + e2 * e2);
+    const T qq = D.finish();
     q = q + qq;
     const int r = y * pitch + x, fs = Ly * pitch;
-    pl[r] = d01;
-    pl[fs + r] = d02;
-    pl[2 * fs + r] = d12;
-    pl[3 * fs + r] = {e0, e1};
+    pl[r] = D.d01;
+    pl[fs + r] = D.d02;
+    pl[2 * fs + r] = D.d12;
+    pl[3 * fs + r] = {D.e0, D.e1};
   }
   const T v[2] = {fsum, q};
   float2 o[2];

@@ -211,6 +211,35 @@ __device__ __forceinline__ void add_to_A_F(cx<T> (&A)[9], T& fs, const cx<T> (&f
   fs = fs + ((fu[0].re + fu[4].re + fu[8].re) + (bu[0].re + bu[4].re + bu[8].re));
 }
 
+// A - A^dagger of add_to_A's A by its upper elements and imaginary diagonal (half of it), without
+// A: nine reals fewer to add per direction, and no pass over the elements afterwards.
+template <class T>
+struct AntiHermSum {
+  cx<T> d01, d02, d12;
+  T e0, e1, e2;
+  // one direction's U_nu(x - nu) - U_nu(x), both as full matrices
+  __device__ __forceinline__ void add(const cx<T> (&fu)[9], const cx<T> (&bu)[9], bool first) {
+    const cx<T> x01 = csub(csub(bu[1], fu[1]), cconj(csub(bu[3], fu[3])));
+    const cx<T> x02 = csub(csub(bu[2], fu[2]), cconj(csub(bu[6], fu[6])));
+    const cx<T> x12 = csub(csub(bu[5], fu[5]), cconj(csub(bu[7], fu[7])));
+    const T y0 = bu[0].im - fu[0].im, y1 = bu[4].im - fu[4].im, y2 = bu[8].im - fu[8].im;
+    d01 = first ? x01 : cadd(d01, x01);
+    d02 = first ? x02 : cadd(d02, x02);
+    d12 = first ? x12 : cadd(d12, x12);
+    e0 = first ? y0 : e0 + y0;
+    e1 = first ? y1 : e1 + y1;
+    e2 = first ? y2 : e2 + y2;
+  }
+  // makes it Delta (the trace removed, the diagonal whole); returns Tr[Delta Delta^dagger]
+  __device__ __forceinline__ T finish() {
+    const T tr = (e0 + e1 + e2) * T(1.0 / 3.0);
+    e0 = T(2) * (e0 - tr);
+    e1 = T(2) * (e1 - tr);
+    e2 = T(2) * (e2 - tr);
+    return T(2) * (cnorm2(d01) + cnorm2(d02) + cnorm2(d12)) + (e0 * e0 + e1 * e1 + e2 * e2);
+  }
+};
+
 // Tr[Delta Delta^dagger] with Delta = A - A^dagger - (1/3) Tr(A - A^dagger)
 template <class T>
 __device__ __forceinline__ T theta_site(const cx<T> (&A)[9]) {
@@ -228,6 +257,17 @@ __device__ __forceinline__ T theta_site(const cx<T> (&A)[9]) {
 #pragma unroll
   for (int e = 0; e < 9; ++e) q = q + (D[e].re * D[e].re + D[e].im * D[e].im);
   return q;
+}
+
+// D of one direction and F += Re Tr f + Re Tr b
+template <class T, int NE>
+__device__ __forceinline__ void add_to_D_F(AntiHermSum<T>& D, T& fs, const cx<T> (&f)[NE], const cx<T> (&b)[NE],
+                                           bool first) {
+  cx<T> fu[9], bu[9];
+  to_full(f, fu);
+  to_full(b, bu);
+  D.add(fu, bu, first);
+  fs = fs + ((fu[0].re + fu[4].re + fu[8].re) + (bu[0].re + bu[4].re + bu[8].re));
 }
 
 // F and Tr[Delta Delta^dagger] of a site just updated, from K' = G K (K of Eq. (5) before
@@ -359,7 +399,7 @@ struct FasdArgs {
   char* links;            // link storage (FP32-12 or FP64-18) of the lattice
   LatDev lat;
   void* kbuf;             // 4 complex fields, [f][t][z][y][x]
-  char* gbuf;             // g(x): rows 0 and 1, 2 * 3 complex elements, planes [w][lexi]
+  char* gbuf;             // g(x): rows 0 and 1 (FP32), 0 to 2 (FP64), planes [w][lexi]
   float2* plane_F;        // per (z, t) plane, as pairs (hi, lo)
   float2* plane_th;
   const int* unit_planes; // n_units + 1 plane boundaries
@@ -496,8 +536,11 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
       su3_update<T, REPRO, FORM>(K, G, a.omega, kCheckGK && measure_now);
       if (kCheckGK && measure_now) site_check_from_GK(K, fs, q);
       cx<T> A[9];
+      AntiHermSum<T> D{};
+      if constexpr (REPRO) {
 #pragma unroll
-      for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
+        for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
+      }
 #pragma unroll 1
       for (int mu = 0; mu < 4; ++mu) {
         cx<T> f[NE], b[NE];
@@ -509,11 +552,17 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
           reunit<REPRO>(f);
           reunit<REPRO>(b);
         }
-        if (!kCheckGK && mu < ND && measure_now) add_to_A_F(A, fs, f, b);
+        if (!kCheckGK && mu < ND && measure_now) {
+          if constexpr (REPRO) add_to_A_F(A, fs, f, b);
+          else add_to_D_F(D, fs, f, b, false);
+        }
         St::store(base, V, mu, idx_f, f);
         St::store(base, V, mu, idx_b[mu], b);
       }
-      if (!kCheckGK && measure_now) q = theta_site(A);
+      if (!kCheckGK && measure_now) {
+        if constexpr (REPRO) q = theta_site(A);
+        else q = D.finish();
+      }
     }
   }
   if (measure_now) {
@@ -551,11 +600,11 @@ __global__ void __launch_bounds__(256) k_measure(MeasureArgs a) {
     const Site s = site_of_slice(lat, p, tile.y, h3);
     const char* base = a.links + lat.off_bytes;
     const int idx_f = p * lat.Vh + h;
-    cx<T> A[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
     T fs = T(0);
     if constexpr (sizeof(T) == 4) {
+      cx<T> A[9];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
       // FP32: issue all 2 nd link loads before any arithmetic (memory-level parallelism)
       cx<T> f[ND][NE], b[ND][NE];
 #pragma unroll
@@ -567,17 +616,20 @@ __global__ void __launch_bounds__(256) k_measure(MeasureArgs a) {
       for (int nu = 0; nu < ND; ++nu) {
         add_to_A_F(A, fs, f[nu], b[nu]);
       }
+      q = theta_site(A);
     } else {
+      // FP64: about 160 instructions of its pipe a site instead of 300 (two of them divisions)
+      AntiHermSum<T> D;
 #pragma unroll
       for (int nu = 0; nu < ND; ++nu) {
         cx<T> f[NE], b[NE];
         St::load(base, lat.V, nu, idx_f, f);
         St::load(base, lat.V, nu, (1 - p) * lat.Vh + (int)(back_lexi(lat, s, nu) >> 1), b);
-        add_to_A_F(A, fs, f, b);
+        add_to_D_F(D, fs, f, b, nu == 0);
       }
+      q = D.finish();
     }
     fsum = fs;
-    q = theta_site(A);
   }
   const T v[2] = {fsum, q};
   float2 o[2];
