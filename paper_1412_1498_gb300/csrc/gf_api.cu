@@ -6,7 +6,8 @@
 // the even-site theta pass for the undecided units; the loop finish) that read and
 // update a small DevState in device memory, so that a captured CUDA graph of many
 // sweeps needs no host decision between them.  The host synchronises once per graph
-// replay to read the number of still-active convergence units.
+// replay to read the number of still-active convergence units.  Handles with several
+// units and few sites run their loop in one cooperative kernel instead (gf_loop.cuh).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,6 +29,7 @@ void launch_sweep_fp32_pipe(int nd, const SweepArgs& a, int n_tiles, int threads
 void launch_measure_fp32_pipe(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s);
 cudaError_t prepare_sweep_pipe();
 cudaError_t prepare_loop();
+cudaError_t prepare_sweep_split();
 cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t s);
 int sweep_pipe_grid(int nd, int threads, int n_tiles);
 void launch_sweep_dir(int storage, int nd, const SweepArgs& a, int n_tiles, cudaStream_t s);
@@ -478,6 +480,7 @@ SweepArgs sweep_args(gf_handle* h, int parity, bool loop, int reverse) {
   a.level = 1;
   a.dep = h->n_units == 1;
   a.dir = h->cur == 0 && dir_kernel_serves(h);
+  a.tile_sites = h->tile;
   a.omega = h->relax;
   return a;
 }
@@ -1322,6 +1325,7 @@ int gf_create_batch(int n_lat, const int* dims, int gauge, int storage, int flag
   {
     cudaError_t e = prepare_sweep_pipe();
     if (e == cudaSuccess) e = prepare_loop();
+    if (e == cudaSuccess && (h->flags & GF_FLAG_MIXED)) e = prepare_sweep_split();
     if (e != cudaSuccess) return bail(GF_ECUDA, std::string("sweep kernel set-up: ") + cudaGetErrorString(e));
   }
   const Layout& L = h->L;

@@ -3,9 +3,25 @@
 
 namespace gf {
 
-void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s) {
-  if (nd == 4) k_or_sweep_split<4><<<n_tiles, threads, 0, s>>>(a);
-  else k_or_sweep_split<3><<<n_tiles, threads, 0, s>>>(a);
+// Shared-memory opt-in of the staged sweep (outside any stream capture).
+cudaError_t prepare_sweep_split() {
+  const int bytes = kSplitWords * kSplitBlock * (int)sizeof(float4);
+  cudaError_t e = cudaFuncSetAttribute(k_or_sweep_split<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_or_sweep_split<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
+}
+
+void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int tile, cudaStream_t s) {
+  const long long link_bytes = 2LL * n_tiles * tile * 4 * 144;  // of the units in the tile table
+  if (link_bytes > (96LL << 20) && tile >= kSplitBlock) {
+    const size_t smem = (size_t)kSplitWords * kSplitBlock * sizeof(float4);
+    if (nd == 4) k_or_sweep_split<4, true><<<n_tiles, kSplitBlock, smem, s>>>(a);
+    else k_or_sweep_split<3, true><<<n_tiles, kSplitBlock, smem, s>>>(a);
+  } else {
+    if (nd == 4) k_or_sweep_split<4, false><<<n_tiles, tile, 0, s>>>(a);
+    else k_or_sweep_split<3, false><<<n_tiles, tile, 0, s>>>(a);
+  }
 }
 
 void launch_measure_split(int nd, const MeasureArgs& a, int n_tiles, int threads, cudaStream_t s) {

@@ -337,6 +337,7 @@ struct SweepArgs {
                            // by blockIdx.x) instead of per tile
   int dep;                 // launch with programmatic stream serialisation (launch_dep)
   int dir;                 // the direction-per-warp kernel (small lattices)
+  int tile_sites;          // sites a tile covers (fewer at the end of a time slice)
   Relax omega;
 };
 

@@ -96,10 +96,19 @@ __device__ __forceinline__ void split_store(char* base, long long V, int mu, int
 #pragma unroll
   for (int w = 0; w < 9; ++w) p[(long long)(w * 4 + mu) * V + idx] = make_float4(u[w].re.hi, u[w].im.hi, u[w].re.lo, u[w].im.lo);
 }
-// Apply phase: the reload of a link is the last use of its line and the store streams
-// out (cache hints ld.global.lu / st.global.cs), so the updated links do not evict the
-// lines that other blocks loaded for their K phase and will reload: 0.537 -> 0.495 ms
-// per 32^4 polish sweep.
+// a link's nine words in shared memory, `stride` words apart
+__device__ __forceinline__ void split_read(const float4* p, int stride, csf (&u)[9]) {
+#pragma unroll
+  for (int w = 0; w < 9; ++w) {
+    const float4 v = p[w * stride];
+    u[w] = {{v.x, v.z}, {v.y, v.w}};
+  }
+}
+__device__ __forceinline__ void split_copy(float4* smem, const float4* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+// (read twice) the reload of a link, the last use of its lines, and the streaming store
 __device__ __forceinline__ void split_load_last(const char* base, long long V, int mu, int idx, csf (&u)[9]) {
   const float4* p = reinterpret_cast<const float4*>(base);
 #pragma unroll
@@ -113,6 +122,7 @@ __device__ __forceinline__ void split_store_stream(char* base, long long V, int 
 #pragma unroll
   for (int w = 0; w < 9; ++w) __stcs(p + (long long)(w * 4 + mu) * V + idx, make_float4(u[w].re.hi, u[w].im.hi, u[w].re.lo, u[w].im.lo));
 }
+
 // hi = (float)x, lo = (float)(x - hi) for the nine elements of a link, by shifts where every
 // part allows it (see widen); one FP64 subtraction a real instead of four instructions of
 // that pipe
@@ -280,8 +290,22 @@ __device__ __forceinline__ float split_theta_site(const acc2 (&A)[18]) {
 }
 
 // ------------------------------------------------------------------------- the sweep
-template <int ND>
-__global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
+// A site's eight links (1152 bytes) do not fit in registers and are needed twice, for K and for
+// the update.  STAGED: each thread copies its site's 72 words to shared memory with cp.async
+// and reads them there (only its own, so there is no barrier); blocks of 64 sites (74 KB), three
+// to an SM: while one updates, the copies of the others are in flight.  Otherwise the links are
+// read twice from memory: the reload is marked as the lines' last use and the stores as
+// streaming, which keeps the lines other blocks will reload in L2.  us a sweep, read twice
+// -> staged: 24^4 (191 MB of links) 161 -> 147, 32^4 (604 MB) 453 -> 426, where the second reads
+// that miss L2 cost DRAM a tenth more traffic; 16^4 (38 MB) 36.3 -> 38.8, 20x12x18x10 36.1 -> 41.0,
+// where the larger number of warps counts.  The line is drawn at 96 MB of links in the tile table
+// (L2 holds 126 MB); 96 or 32 sites a block were slower (24^4 192, 179).
+constexpr int kSplitBlock = 64;
+constexpr int kSplitWords = 72;  // word w of the side (0 forward, 1 backward) link mu: (2 mu + side) 9 + w
+
+template <int ND, bool STAGED>
+__global__ void __launch_bounds__(STAGED ? kSplitBlock : 256, STAGED ? 3 : 1) k_or_sweep_split(SweepArgs a) {
+  extern __shared__ float4 sm[];
   __shared__ double red[64];
   bool reunit_now = a.reunit != 0, measure_now = a.measure != 0;
   if (a.st) {
@@ -293,9 +317,12 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
   const int4 tile = a.tiles[ti];
   if (a.active && a.active[tile.w] != a.level) return;
   const LatDev lat = a.lats[tile.x];
-  const int h3 = tile.z + (int)threadIdx.x;
-  float q = 0.f, fsum = 0.f;
-  if (h3 < lat.V3h) {
+  const int B = (int)blockDim.x;
+  float4* slot = sm + threadIdx.x;
+  float acc_hi[2] = {0.f, 0.f}, acc_lo[2] = {0.f, 0.f};  // this thread's sites of the tile
+#pragma unroll 1
+  for (int h3 = tile.z + (int)threadIdx.x; h3 < tile.z + a.tile_sites && h3 < lat.V3h; h3 += B) {
+    float q = 0.f, fsum = 0.f;
     const int p = a.parity;
     const int h = tile.y * lat.V3h + h3;
     const Site s = site_of_slice(lat, p, tile.y, h3);
@@ -306,6 +333,17 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) idx_b[mu] = (1 - p) * lat.Vh + (int)(back_lexi(lat, s, mu) >> 1);
     const float omega = (float)a.omega.omega;
+    if constexpr (STAGED) {
+      const float4* g = reinterpret_cast<const float4*>(base);
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+        for (int w = 0; w < 9; ++w) {
+          split_copy(slot + (18 * mu + w) * B, g + (long long)(w * 4 + mu) * V + idx_f);
+          split_copy(slot + (18 * mu + 9 + w) * B, g + (long long)(w * 4 + mu) * V + idx_b[mu]);
+        }
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+    }
 
     // K = sum_{mu<nd} U_mu(x) + U_mu(x-mu)^+ with TwoSum on the hi parts
     acc2 K[18];
@@ -314,8 +352,13 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
 #pragma unroll 1
     for (int mu = 0; mu < ND; ++mu) {
       csf f[9], b[9];
-      split_load(base, V, mu, idx_f, f);
-      split_load(base, V, mu, idx_b[mu], b);
+      if constexpr (STAGED) {
+        split_read(slot + 18 * mu * B, B, f);
+        split_read(slot + (18 * mu + 9) * B, B, b);
+      } else {
+        split_load(base, V, mu, idx_f, f);
+        split_load(base, V, mu, idx_b[mu], b);
+      }
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -389,7 +432,8 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
       for (int side = 0; side < 2; ++side) {
         const int idx = side == 0 ? idx_f : idx_b[mu];
         csf u[9];
-        split_load_last(base, V, mu, idx, u);
+        if constexpr (STAGED) split_read(slot + (18 * mu + 9 * side) * B, B, u);
+        else split_load_last(base, V, mu, idx, u);
         cx<float> du[9];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
@@ -415,16 +459,26 @@ __global__ void __launch_bounds__(256) k_or_sweep_split(SweepArgs a) {
           }
           tr[side] = sf_f(u[0].re) + sf_f(u[4].re) + sf_f(u[8].re);
         }
-        split_store_stream(base, V, mu, idx, u);
+        if constexpr (STAGED) split_store(base, V, mu, idx, u);
+        else split_store_stream(base, V, mu, idx, u);
       }
       if (mu < ND && measure_now) fsum = fsum + (tr[0] + tr[1]);
     }
-    if (measure_now) q = split_theta_site(A);
+    if (measure_now) {
+      q = split_theta_site(A);
+      const float v[2] = {fsum, q};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float s2, e2;
+        two_sum(acc_hi[j], v[j], s2, e2);
+        acc_hi[j] = s2;
+        acc_lo[j] = acc_lo[j] + e2;
+      }
+    }
   }
   if (measure_now) {
-    const float v[2] = {fsum, q};
     float2 o[2];
-    block_sum_f32<2>(v, o, reinterpret_cast<float*>(red));
+    block_sum_f32_pairs<2>(acc_hi, acc_lo, o, reinterpret_cast<float*>(red));
     if (threadIdx.x == 0) {
       if (a.part_F) a.part_F[ti] = o[0];
       a.part_theta[ti] = o[1];

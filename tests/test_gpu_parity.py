@@ -608,3 +608,22 @@ def test_small_lattice_equals_batch_member(gf, storage, gauge, dims, form):
     (ua, ia, Fa, ta), (ub, ib, Fb, tb) = res
     assert np.array_equal(ua, ub) and np.array_equal(ia, ib)
     assert abs(Fa - Fb) < 1e-12 and abs(ta - tb) < 1e-12 * max(ta, 1e-3)
+
+
+def test_staged_polish_equals_small_batches_polish(gf):
+    # above 96 MB of links the double-float sweep stages them in shared memory; one of six equal
+    # lattices in a batch above the line (6 x 18 MB of links), one alone below it: the same bits
+    dims = (16, 12, 10, 16)
+    U = fields.smooth_field(dims, 0.02, 97)
+    res = []
+    for n in (1, 6):
+        fx = gf.GaugeFixer([dims] * n, gf.GF_LANDAU, gf.GF_FP32_12, mixed=True)
+        gf.gf_set_mixed_switch(fx.h, 1e3)               # every sweep in double-float
+        for i in range(n):
+            fx.upload(U, i)
+        out = fx.fix(1e-300, 21)
+        res.append((fx.download(n - 1), out["F"][n - 1], out["theta"][n - 1], out["iters"][n - 1]))
+        fx.close()
+    (ua, Fa, ta, ia), (ub, Fb, tb, ib) = res
+    assert ia == ib == 21 and np.array_equal(ua, ub)
+    assert abs(Fa - Fb) < 1e-12 and abs(ta - tb) < 1e-12 * ta
