@@ -509,17 +509,6 @@ __device__ __forceinline__ void to_full(const cx<T> (&e)[NE], cx<T> (&m)[9]) {
   if constexpr (NE == 6) third_row<PLAIN>(e, m + 6);
 }
 
-// Re Tr of a stored link
-template <class T, int NE>
-__device__ __forceinline__ T re_trace(const cx<T> (&e)[NE]) {
-  if constexpr (NE == 9) {
-    return e[0].re + e[4].re + e[8].re;
-  } else {
-    cx<T> u22 = csub(cmul(e[0], e[4]), cmul(e[1], e[3]));  // conj() keeps the real part
-    return e[0].re + e[4].re + u22.re;
-  }
-}
-
 // out rows (NE/3 of them) = G * U, U given by its stored elements
 template <bool PLAIN = false, class T, int NE>
 __device__ __forceinline__ void left_mul(const cx<T> (&G)[9], cx<T> (&e)[NE]) {
@@ -637,11 +626,6 @@ __device__ __forceinline__ Site site_of_slice(const LatDev& lat, int parity, int
   return s;
 }
 
-__device__ __forceinline__ Site site_of(const LatDev& lat, int parity, int h) {
-  const int t = h / lat.V3h;
-  return site_of_slice(lat, parity, t, h - t * lat.V3h);
-}
-
 // lexicographic index of x - mu_hat (periodic)
 __device__ __forceinline__ long long back_lexi(const LatDev& lat, const Site& s, int mu) {
   const long long Lx = lat.L[0], LxLy = Lx * lat.L[1], V3 = LxLy * lat.L[2];
@@ -651,26 +635,6 @@ __device__ __forceinline__ long long back_lexi(const LatDev& lat, const Site& s,
     case 2: return s.z == 0 ? s.lexi + LxLy * (lat.L[2] - 1) : s.lexi - LxLy;
     default: return s.t == 0 ? s.lexi + V3 * (lat.L[3] - 1) : s.lexi - V3;
   }
-}
-
-// parity-split index of the site with lexicographic index lexi
-__device__ __forceinline__ int idx_from_lexi(const LatDev& lat, long long lexi) {
-  long long r = lexi;
-  const int x = (int)(r % lat.L[0]); r /= lat.L[0];
-  const int y = (int)(r % lat.L[1]); r /= lat.L[1];
-  const int z = (int)(r % lat.L[2]);
-  const int t = (int)(r / lat.L[2]);
-  return ((x + y + z + t) & 1) * lat.Vh + (int)(lexi >> 1);
-}
-
-// lexicographic index of lexi + dir * mu_hat (periodic), dir = +1 or -1
-__device__ __forceinline__ long long lexi_step(const LatDev& lat, long long lexi, int mu, int dir) {
-  long long stride = 1;
-  for (int k = 0; k < mu; ++k) stride *= lat.L[k];
-  const int c = (int)((lexi / stride) % lat.L[mu]);
-  const int L = lat.L[mu];
-  if (dir > 0) return c == L - 1 ? lexi - stride * (L - 1) : lexi + stride;
-  return c == 0 ? lexi + stride * (L - 1) : lexi - stride;
 }
 
 // ----------------------------------------------------------------------------------

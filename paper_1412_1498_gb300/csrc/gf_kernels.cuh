@@ -45,9 +45,7 @@ inline Relax relax_of(double omega) {
   }
   return r;
 }
-__device__ __forceinline__ double relax_mu(const Relax&, double) { return 1.0; }
 __device__ __forceinline__ double relax_q(const Relax& w, double) { return w.kappa; }
-__device__ __forceinline__ float relax_mu(const Relax& w, float) { return w.mu; }
 __device__ __forceinline__ float relax_q(const Relax& w, float) { return w.q; }
 
 template <class T, bool REPRO, int FORM>
@@ -70,7 +68,7 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
       // (a first normalisation off by an ulp shifts kappa by as much, unlike the second one it
       // leaves g unitary: the plain FP32 instruction serves)
       T rn;
-      if constexpr (sizeof(T) == 4) rn = rsqrtf(n2) * relax_mu(w, T(0));
+      if constexpr (sizeof(T) == 4) rn = rsqrtf(n2) * w.mu;
       else rn = gf_rsqrt(n2);
       const cx<T> a1 = {gf_fma(alpha.re, rn, relax_q(w, T(0))), -alpha.im * rn};
       const cx<T> b1 = {beta.re * rn, -beta.im * rn};
@@ -189,18 +187,9 @@ __device__ __forceinline__ void add_to_K(cx<T> (&K)[9], const cx<T> (&f)[NE], co
     }
 }
 
-// A += U_nu(x - nu) - U_nu(x)  (Eq. (3), one direction)
-template <class T, int NE>
-__device__ __forceinline__ void add_to_A(cx<T> (&A)[9], const cx<T> (&f)[NE], const cx<T> (&b)[NE]) {
-  cx<T> fu[9], bu[9];
-  to_full(f, fu);
-  to_full(b, bu);
-#pragma unroll
-  for (int e = 0; e < 9; ++e) A[e] = cadd(A[e], csub(bu[e], fu[e]));
-}
-
-// add_to_A and F += Re Tr f + Re Tr b from the same full matrices (Re Tr of a 12-real
-// link is e0 + e4 + Re(e0 e4 - e1 e3), the (2,2) element of its rebuilt third row)
+// A += U_nu(x - nu) - U_nu(x) (Eq. (3), one direction) and F += Re Tr f + Re Tr b from the
+// same full matrices (Re Tr of a 12-real link is e0 + e4 + Re(e0 e4 - e1 e3), the (2,2)
+// element of its rebuilt third row)
 template <class T, int NE>
 __device__ __forceinline__ void add_to_A_F(cx<T> (&A)[9], T& fs, const cx<T> (&f)[NE], const cx<T> (&b)[NE]) {
   cx<T> fu[9], bu[9];
@@ -211,7 +200,7 @@ __device__ __forceinline__ void add_to_A_F(cx<T> (&A)[9], T& fs, const cx<T> (&f
   fs = fs + ((fu[0].re + fu[4].re + fu[8].re) + (bu[0].re + bu[4].re + bu[8].re));
 }
 
-// A - A^dagger of add_to_A's A by its upper elements and imaginary diagonal (half of it), without
+// A - A^dagger of add_to_A_F's A by its upper elements and imaginary diagonal (half of it), without
 // A: nine reals fewer to add per direction, and no pass over the elements afterwards.
 template <class T>
 struct AntiHermSum {
