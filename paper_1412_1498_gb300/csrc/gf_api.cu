@@ -30,7 +30,7 @@ void launch_measure_fp32_pipe(int nd, const MeasureArgs& a, int n_tiles, int thr
 cudaError_t prepare_sweep_pipe();
 cudaError_t prepare_loop();
 cudaError_t prepare_sweep_split();
-cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t s);
+cudaError_t launch_loop(int storage, int nd, LoopArgs a, cudaStream_t s);
 int sweep_pipe_grid(int nd, int threads, int n_tiles);
 void launch_sweep_dir(int storage, int nd, const SweepArgs& a, int n_tiles, cudaStream_t s);
 void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int threads, cudaStream_t s);
@@ -756,10 +756,11 @@ int run_phase(gf_handle* h, double eps, int budget, int* done) {
 }
 
 // Whether a call's sweeps run in the one-kernel loop (gf_loop.cuh, which says where the line
-// lies): several units, FP32 storage with full or 12-real links, the default kernel and block
-// size, no history, and few enough sites, tiles and units.
+// lies): several units, FP32 storage with full or 12-real links, the first-order form, the
+// default kernel and block size, no history, and few enough sites, tiles and units.
 bool loop_kernel_serves(const gf_handle* h) {
   if (h->cur != 0 || (h->storage != GF_FP32_12 && h->storage != GF_FP32_18)) return false;
+  if (h->form != GF_OR_FIRST_ORDER) return false;
   if (h->variant != GF_SWEEP_AUTO || h->tile != kLoopThreads || h->hist || h->n_units == 1 || h->n_units > kLoopUnits) return false;
   long long sites = 0;
   for (const LatDev& lat : h->lats) sites += lat.V;
@@ -811,7 +812,7 @@ int run_phase_loop(gf_handle* h, double eps, int budget, int* done) {
   a.nd = h->nd;
   a.omega = h->relax;
   for (int before = offset - 1;;) {
-    const cudaError_t e = launch_loop(h->storage, h->nd, h->form, a, h->stream);
+    const cudaError_t e = launch_loop(h->storage, h->nd, a, h->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge && before == offset - 1) {
       cudaGetLastError();  // fewer SMs than the device has (a partitioned context): launches instead
       return run_phase(h, eps, budget, done);
@@ -1526,11 +1527,10 @@ int gf_or_sweep(gf_handle* h, int parity, double omega) {
   if (parity < 0 || parity > 2) return fail(h, GF_EINVAL, "parity must be 0, 1 or 2");
   if (!(omega >= 1.0 && omega < 2.0)) return fail(h, GF_EINVAL, "omega must lie in [1, 2)");
   const int st = cur_storage(h);
-  const Relax relax = omega == h->omega ? h->relax : relax_of(omega);
   for (int p = 0; p < 2; ++p) {
     if (parity != 2 && p != parity) continue;
     SweepArgs a = sweep_args(h, p, false, p);
-    a.omega = relax;
+    a.omega = relax_of(omega);
     launch_sweep(st, h->nd, h->repro, h->variant, a, h->n_tiles, h->tile, h->stream);
     GF_CK_LAUNCH(h);
   }

@@ -23,8 +23,12 @@
 // The arithmetic helpers below spell out every complex operation in a fixed order.  The
 // matrix products come in two forms: PLAIN = true sums the products as a plain C
 // implementation does and, compiled with -fmad=false (the "reproducible" FP64 kernels),
-// performs exactly its IEEE operations; PLAIN = false (every other kernel) accumulates
-// with chains of fused multiply-adds.
+// performs exactly its IEEE operations; PLAIN = false accumulates with chains of fused
+// multiply-adds (the other FP64 kernels, the double-float polish, Fourier acceleration).
+// The FP32 overrelaxation sweeps, their checks and the FP32 F / theta pass take the plain
+// form too (kPlain), contracted as nvcc contracts it, the same in each of them: rounding
+// grows along a run's slow modes, theta of a few thousand FP32 sites moves by 1e-6 of itself
+// with any other rounding, and with it the sweeps that a run near a saddle takes.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -173,8 +177,7 @@ __device__ __forceinline__ double gf_fma(double a, double b, double c) { return 
 // an add per component), and a sum that starts at zero keeps its first addition: a product
 // of 3 x 3 matrices is 108 instructions with these where it was 162.  FP64 sweeps issue
 // nothing but such chains on a pipe of two lanes per SM: 16^4 FP64-18 half-sweep 139.6 ->
-// 97.1 us; sweeps of lattices that L2 holds are bound by issue slots.  One rounding per
-// product instead of two.
+// 97.1 us.  One rounding per product instead of two.
 template <class T>
 __device__ __forceinline__ void cmac(cx<T>& acc, cx<T> x, cx<T> y) {
   acc.re = gf_fma(x.re, y.re, acc.re);
@@ -199,11 +202,8 @@ __device__ __forceinline__ cx<T> cmul_conj_fma(cx<T> x, cx<T> y) {
   return {gf_fma(x.im, y.im, x.re * y.re), gf_fma(-x.re, y.im, x.im * y.re)};
 }
 
-// x^(-1/2) with the error of a rounding.  The hardware's FP32 reciprocal square root is off
-// by up to 2 units in the last place and not evenly to both sides; as the normalisation of
-// an SU(2) element that makes every g stretch the links it is applied to.  One Newton step
-// removes it: F of FP32 fields after 20 sweeps was off by 3e-6 to 4e-6 (32^4, 24^4), now by
-// less than 1e-7, in the same time.
+// x^(-1/2) with the error of a rounding: FP32 by one Newton step on the hardware's reciprocal
+// square root, which is off by up to 1.2e-7 of it.
 __device__ __forceinline__ double gf_rsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float gf_rsqrt(float x) {
   const float r = rsqrtf(x);
@@ -255,6 +255,10 @@ __device__ __forceinline__ float narrow_shift(double x) {  // to nearest even
   r += rest > 0x80000000u ? 1u : (rest == 0x80000000u ? (r & 1u) : 0u);
   return __uint_as_float((hi & 0x80000000u) | ((m | lo) == 0u ? 0u : r));
 }
+
+// Which form the sweeps' products take (see the top of this file)
+template <class T, bool REPRO = false>
+constexpr bool kPlain = REPRO || sizeof(T) == 4;
 
 template <class T>
 __device__ __forceinline__ T gf_sqrt(T x);

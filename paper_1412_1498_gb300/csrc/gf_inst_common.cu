@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(256) k_reunit(char* links, LatDev lat) {
   const int mu = (int)(i / lat.V), idx = (int)(i % lat.V);
   cx<T> e[St::NE];
   St::load(links + lat.off_bytes, lat.V, mu, idx, e);
-  reunit(e);
+  reunit<kPlain<T>>(e);
   St::store(links + lat.off_bytes, lat.V, mu, idx, e);
 }
 

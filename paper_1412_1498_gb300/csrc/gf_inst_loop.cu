@@ -8,14 +8,9 @@ namespace {
 constexpr int kMaxDev = 64;
 int g_loop_grid[kMaxDev];  // blocks that fit the device together (every instance's minimum)
 
-const void* loop_kernel(int storage, int nd, int form) {
-#define GF_PICK(S)                                                                              \
-  (nd == 4 ? (form == GF_OR_FIRST_ORDER ? (const void*)k_loop<S, 4, GF_OR_FIRST_ORDER>          \
-                                        : (const void*)k_loop<S, 4, GF_OR_EXACT>)               \
-           : (form == GF_OR_FIRST_ORDER ? (const void*)k_loop<S, 3, GF_OR_FIRST_ORDER>          \
-                                        : (const void*)k_loop<S, 3, GF_OR_EXACT>))
-  return storage == GF_FP32_12 ? GF_PICK(GF_FP32_12) : GF_PICK(GF_FP32_18);
-#undef GF_PICK
+const void* loop_kernel(int storage, int nd) {
+  if (storage == GF_FP32_12) return nd == 4 ? (const void*)k_loop<GF_FP32_12, 4> : (const void*)k_loop<GF_FP32_12, 3>;
+  return nd == 4 ? (const void*)k_loop<GF_FP32_18, 4> : (const void*)k_loop<GF_FP32_18, 3>;
 }
 }  // namespace
 
@@ -29,18 +24,17 @@ cudaError_t prepare_loop() {
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   int least = 1 << 30;
   for (int st : {GF_FP32_12, GF_FP32_18})
-    for (int nd : {3, 4})
-      for (int form : {GF_OR_FIRST_ORDER, GF_OR_EXACT}) {
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, loop_kernel(st, nd, form), kLoopThreads, 0);
-        if (e != cudaSuccess) return e;
-        if (per_sm < least) least = per_sm;
-      }
+    for (int nd : {3, 4}) {
+      int per_sm = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, loop_kernel(st, nd), kLoopThreads, 0);
+      if (e != cudaSuccess) return e;
+      if (per_sm < least) least = per_sm;
+    }
   g_loop_grid[dev] = least * sms;
   return cudaSuccess;
 }
 
-cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t s) {
+cudaError_t launch_loop(int storage, int nd, LoopArgs a, cudaStream_t s) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -48,7 +42,7 @@ cudaError_t launch_loop(int storage, int nd, int form, LoopArgs a, cudaStream_t 
   if (most <= 0) return cudaErrorInvalidConfiguration;
   const int grid = a.n_tiles < most ? a.n_tiles : most;
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel(loop_kernel(storage, nd, form), dim3(grid), dim3(kLoopThreads), args, 0, s);
+  return cudaLaunchCooperativeKernel(loop_kernel(storage, nd), dim3(grid), dim3(kLoopThreads), args, 0, s);
 }
 
 }  // namespace gf

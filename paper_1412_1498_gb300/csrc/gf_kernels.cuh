@@ -15,38 +15,16 @@ namespace gf {
 //   Re(a alpha) + Re(b beta) for R|_(i,j) = [[a, b], [-conj b, conj a]], maximal at
 //   (a, b) = conj(alpha, beta) / |(alpha, beta)|; R = 1 when alpha = beta = 0.
 // REPRO: IEEE divisions in the order of a plain C implementation; otherwise one
-// reciprocal square root and multiplications.
+// reciprocal square root and multiplications (FP32: the hardware's, as it comes).
 // ----------------------------------------------------------------------------------
 // The overrelaxation parameter as the kernels take it.  To first order g^omega = 1 + omega
-// (g - 1), renormalised, is (a, b) -> mu (a + kappa, b) with kappa = (1 - omega) / omega and
-// any mu > 0.  mu is chosen (relax_of) so that q = mu kappa is a float to 1e-11: omega
-// rounded to FP32 changes the rate at which theta falls, by 2e-6 of theta after 24 sweeps.
+// (g - 1), renormalised, is (a, b) -> (a + kappa, b) up to a factor that the normalisation
+// removes, with kappa = (1 - omega) / omega: the form of the FP64 update.
 struct Relax {
   double omega, kappa;
-  float mu, q;
 };
 
-inline Relax relax_of(double omega) {
-  Relax r;
-  r.omega = omega;
-  r.kappa = (1.0 - omega) / omega;
-  r.mu = 1.f;
-  r.q = (float)r.kappa;
-  if (r.kappa == 0.0) return r;
-  double best = 1.0;
-  for (int k = 0; k < 4096 && best > 1e-11; ++k) {
-    const double mu = 1.0 + k / 4096.0, q = mu * r.kappa;
-    const double e = (double)(float)q / q - 1.0, err = e < 0.0 ? -e : e;
-    if (err < best) {
-      best = err;
-      r.mu = (float)mu;
-      r.q = (float)q;
-    }
-  }
-  return r;
-}
-__device__ __forceinline__ double relax_q(const Relax& w, double) { return w.kappa; }
-__device__ __forceinline__ float relax_q(const Relax& w, float) { return w.q; }
+inline Relax relax_of(double omega) { return {omega, (1.0 - omega) / omega}; }
 
 template <class T, bool REPRO, int FORM>
 __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j, const Relax& w,
@@ -63,16 +41,12 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
       a = {alpha.re / n, -alpha.im / n};
       b = {beta.re / n, -beta.im / n};
     }
-  } else if constexpr (FORM == GF_OR_FIRST_ORDER) {
+  } else if constexpr (FORM == GF_OR_FIRST_ORDER && sizeof(T) == 8) {
     if (n2 > T(0)) {
-      // (a first normalisation off by an ulp shifts kappa by as much, unlike the second one it
-      // leaves g unitary: the plain FP32 instruction serves)
-      T rn;
-      if constexpr (sizeof(T) == 4) rn = rsqrtf(n2) * w.mu;
-      else rn = gf_rsqrt(n2);
-      const cx<T> a1 = {gf_fma(alpha.re, rn, relax_q(w, T(0))), -alpha.im * rn};
+      const T rn = gf_rsqrt(n2);
+      const cx<T> a1 = {gf_fma(alpha.re, rn, w.kappa), -alpha.im * rn};
       const cx<T> b1 = {beta.re * rn, -beta.im * rn};
-      // |a1 + ...|^2 >= mu^2 (1 - |kappa|)^2 > 0
+      // |a1 + ...|^2 >= (1 - |kappa|)^2 > 0
       const T rm = gf_rsqrt(((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im);
       a = cscale(a1, rm);
       b = cscale(b1, rm);
@@ -80,7 +54,9 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
     return;
   } else {
     if (n2 > T(0)) {
-      const T rn = gf_rsqrt(n2);
+      T rn;
+      if constexpr (sizeof(T) == 4) rn = rsqrtf(n2);
+      else rn = gf_rsqrt(n2);
       a = {alpha.re * rn, -alpha.im * rn};
       b = {beta.re * rn, -beta.im * rn};
     }
@@ -89,10 +65,17 @@ __device__ __forceinline__ void su2_maximiser(const cx<T> (&K)[9], int i, int j,
     // g^omega to first order: 1 + omega (g - 1), renormalised onto SU(2)
     const cx<T> a1 = {(T(1) - omega) + omega * a.re, omega * a.im};
     const cx<T> b1 = {omega * b.re, omega * b.im};
-    const T m = gf_sqrt(((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im);
-    if (m > T(0)) {
-      a = {a1.re / m, a1.im / m};
-      b = {b1.re / m, b1.im / m};
+    const T m2 = ((a1.re * a1.re + a1.im * a1.im) + b1.re * b1.re) + b1.im * b1.im;
+    if constexpr (REPRO) {
+      const T m = gf_sqrt(m2);
+      if (m > T(0)) {
+        a = {a1.re / m, a1.im / m};
+        b = {b1.re / m, b1.im / m};
+      }
+    } else if (m2 > T(0)) {
+      const T rm = rsqrtf(m2);
+      a = cscale(a1, rm);
+      b = cscale(b1, rm);
     }
   } else {
     // exact power: R = cos(phi) + i sin(phi) n.sigma  ->  cos(omega phi) + i sin(omega phi) n.sigma
@@ -127,16 +110,17 @@ __device__ __forceinline__ void su2_left_mul(cx<T> (&M)[9], int i, int j, cx<T> 
 
 // G = product of the three subgroup maximisers for K (Cabibbo-Marinari order (0,1),
 // (0,2), (1,2)), K rotated after each one.
-// The first product R1 * 1 is R1 itself, and outside the reproducible arithmetic the
-// second one, R2 R1, skips the products with R1's zeros and its 1 (a compiler may not: 0 x
-// is not 0 for every x).  K is left as R2 R1 K unless rotate_last asks for the third
+// The first product R1 * 1 is R1 itself (x * 1 = x, x + 0 = x: the values of the plain
+// sequence), and in the chains of FP64 the second one, R2 R1, skips the products with R1's
+// zeros and its 1 (a compiler may not: 0 x is not 0 for every x).  K is left as R2 R1 K unless rotate_last asks for the third
 // rotation too, which leaves K = G K (used by the fused check, see site_check_from_GK).
 template <class T, bool REPRO, int FORM>
 __device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], const Relax& omega,
                                            bool rotate_last = false) {
+  constexpr bool P = kPlain<T, REPRO>;
   cx<T> a, b;
   su2_maximiser<T, REPRO, FORM>(K, 0, 1, omega, a, b);
-  su2_left_mul<REPRO>(K, 0, 1, a, b);
+  su2_left_mul<P>(K, 0, 1, a, b);
 #pragma unroll
   for (int e = 0; e < 9; ++e) G[e] = {T(0), T(0)};
   G[0] = a;
@@ -145,9 +129,9 @@ __device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], const R
   G[4] = cconj(a);
   G[8] = {T(1), T(0)};
   su2_maximiser<T, REPRO, FORM>(K, 0, 2, omega, a, b);
-  su2_left_mul<REPRO>(K, 0, 2, a, b);
-  if constexpr (REPRO) {
-    su2_left_mul<REPRO>(G, 0, 2, a, b);
+  su2_left_mul<P>(K, 0, 2, a, b);
+  if constexpr (P) {
+    su2_left_mul<P>(G, 0, 2, a, b);
   } else {
     // row 0 = (a G00, a G01, b), row 2 = (-conj(b) G00, -conj(b) G01, conj(a)); G12 = 0
     const cx<T> nb = cneg(b);
@@ -159,15 +143,15 @@ __device__ __forceinline__ void su3_update(cx<T> (&K)[9], cx<T> (&G)[9], const R
     G[2] = b;
   }
   su2_maximiser<T, REPRO, FORM>(K, 1, 2, omega, a, b);
-  if constexpr (REPRO) {
-    su2_left_mul<REPRO>(G, 1, 2, a, b);
+  if constexpr (P) {
+    su2_left_mul<P>(G, 1, 2, a, b);
   } else {
     const cx<T> g22 = G[8];
-    su2_left_mul<REPRO>(G, 1, 2, a, b);  // (its third column is replaced: dead code)
+    su2_left_mul<P>(G, 1, 2, a, b);  // (its third column is replaced: dead code)
     G[5] = cmul_fma(b, g22);
     G[8] = cmul_conj_fma(g22, a);
   }
-  if (rotate_last) su2_left_mul<REPRO>(K, 1, 2, a, b);
+  if (rotate_last) su2_left_mul<P>(K, 1, 2, a, b);
 }
 
 // K += U_mu(x) + U_mu(x - mu)^dagger (in-place form of Eq. (5)); `first` direction: K =
@@ -176,8 +160,8 @@ template <class T, int NE>
 __device__ __forceinline__ void add_to_K(cx<T> (&K)[9], const cx<T> (&f)[NE], const cx<T> (&b)[NE],
                                          bool first = false) {
   cx<T> fu[9], bu[9];
-  to_full(f, fu);
-  to_full(b, bu);
+  to_full<kPlain<T>>(f, fu);
+  to_full<kPlain<T>>(b, bu);
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -193,8 +177,8 @@ __device__ __forceinline__ void add_to_K(cx<T> (&K)[9], const cx<T> (&f)[NE], co
 template <class T, int NE>
 __device__ __forceinline__ void add_to_A_F(cx<T> (&A)[9], T& fs, const cx<T> (&f)[NE], const cx<T> (&b)[NE]) {
   cx<T> fu[9], bu[9];
-  to_full(f, fu);
-  to_full(b, bu);
+  to_full<kPlain<T>>(f, fu);
+  to_full<kPlain<T>>(b, bu);
 #pragma unroll
   for (int e = 0; e < 9; ++e) A[e] = cadd(A[e], csub(bu[e], fu[e]));
   fs = fs + ((fu[0].re + fu[4].re + fu[8].re) + (bu[0].re + bu[4].re + bu[8].re));
@@ -504,11 +488,11 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
       for (int e = 0; e < 9; ++e) A[e] = {T(0), T(0)};
 #pragma unroll
       for (int mu = 0; mu < 4; ++mu) {
-        left_mul<REPRO>(G, f[mu]);
-        right_mul_dag<REPRO>(b[mu], G);
+        left_mul<kPlain<T, REPRO>>(G, f[mu]);
+        right_mul_dag<kPlain<T, REPRO>>(b[mu], G);
         if (reunit_now) {
-          reunit<REPRO>(f[mu]);
-          reunit<REPRO>(b[mu]);
+          reunit<kPlain<T, REPRO>>(f[mu]);
+          reunit<kPlain<T, REPRO>>(b[mu]);
         }
         if (!kCheckGK && mu < ND && measure_now) add_to_A_F(A, fs, f[mu], b[mu]);
         St::store(base, V, mu, idx_f, f[mu]);
@@ -536,11 +520,11 @@ __global__ void __launch_bounds__(256) k_or_sweep(SweepArgs a) {
         cx<T> f[NE], b[NE];
         St::load(base, V, mu, idx_f, f);
         St::load(base, V, mu, idx_b[mu], b);
-        left_mul<REPRO>(G, f);
-        right_mul_dag<REPRO>(b, G);
+        left_mul<kPlain<T, REPRO>>(G, f);
+        right_mul_dag<kPlain<T, REPRO>>(b, G);
         if (reunit_now) {
-          reunit<REPRO>(f);
-          reunit<REPRO>(b);
+          reunit<kPlain<T, REPRO>>(f);
+          reunit<kPlain<T, REPRO>>(b);
         }
         if (!kCheckGK && mu < ND && measure_now) {
           if constexpr (REPRO) add_to_A_F(A, fs, f, b);

@@ -17,7 +17,9 @@
 // tiles | their totals and FINISH_LOOP's decisions |.  "|" is a barrier (about 2.5 us on this
 // GPU: the fence, the arrival and a poll are round trips to L2 each).  Per-site arithmetic, tile
 // sums and the order of the totals are those of the kernels for other handles: the same bits.
-// Links are read past L1, which other SMs' stores do not reach.
+// Links are read past L1, which other SMs' stores do not reach.  Only the first-order form of the
+// overrelaxation runs here: nvcc contracts the exact form's products otherwise than in the
+// sweep kernels, and the links would not be the same bits.
 //
 // Coulomb gauge FP32-12, us a sweep, launches -> this kernel: 8^3x16 21.2 -> 14.8, 12^3x16
 // 21.8 -> 15.2, 16^3x32 32.4 -> 26.1 (above that the pipelined kernels' bandwidth counts for
@@ -172,7 +174,7 @@ __device__ __forceinline__ void loop_unit_sum(const float2* const (&p)[NV], int 
   __syncthreads();
 }
 
-template <int S, int ND, int FORM>
+template <int S, int ND>
 __global__ void __launch_bounds__(kLoopThreads, 2) k_loop(LoopArgs a) {
   using St = Store<S>;
   using Ld = LoopStore<S>;
@@ -224,15 +226,15 @@ __global__ void __launch_bounds__(kLoopThreads, 2) k_loop(LoopArgs a) {
           }
 #pragma unroll
           for (int mu = 0; mu < ND; ++mu) add_to_K(K, f[mu], b[mu], mu == 0);
-          su3_update<float, false, FORM>(K, Gx, a.omega, measure_now);
+          su3_update<float, false, GF_OR_FIRST_ORDER>(K, Gx, a.omega, measure_now);
           if (measure_now) site_check_from_GK(K, v[0], v[1]);
 #pragma unroll
           for (int mu = 0; mu < 4; ++mu) {
-            left_mul(Gx, f[mu]);
-            right_mul_dag(b[mu], Gx);
+            left_mul<true>(Gx, f[mu]);
+            right_mul_dag<true>(b[mu], Gx);
             if (reunit_now) {
-              reunit(f[mu]);
-              reunit(b[mu]);
+              reunit<true>(f[mu]);
+              reunit<true>(b[mu]);
             }
             St::store(base, V, mu, s.idx_f, f[mu]);
             St::store(base, V, mu, s.idx_b[mu], b[mu]);

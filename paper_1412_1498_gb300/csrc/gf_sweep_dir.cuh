@@ -103,11 +103,11 @@ __global__ void __launch_bounds__(kDirThreads, dir_min_blocks<S>()) k_or_sweep_d
     cx<T> G[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) G[e] = {gs[2 * e][lane], gs[2 * e + 1][lane]};
-    left_mul(G, f);
-    right_mul_dag(b, G);
+    left_mul<kPlain<T>>(G, f);
+    right_mul_dag<kPlain<T>>(b, G);
     if (reunit_now) {
-      reunit(f);
-      reunit(b);
+      reunit<kPlain<T>>(f);
+      reunit<kPlain<T>>(b);
     }
     if (!kCheckGK && mu < ND && measure_now) {
       cx<T> fu[9], bu[9];

@@ -127,11 +127,11 @@ __global__ void __launch_bounds__(256) k_or_sweep_pipe(SweepArgs a) {
           cx<float> f[6], b[6];
           pipe_read(slot, B, 3 * mu, f);
           pipe_read(slot, B, 12 + 3 * mu, b);
-          left_mul(G, f);
-          right_mul_dag(b, G);
+          left_mul<true>(G, f);
+          right_mul_dag<true>(b, G);
           if (reunit_now) {
-            reunit(f);
-            reunit(b);
+            reunit<true>(f);
+            reunit<true>(b);
           }
 #pragma unroll
           for (int w = 0; w < 3; ++w) {

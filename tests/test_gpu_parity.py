@@ -627,3 +627,26 @@ def test_staged_polish_equals_small_batches_polish(gf):
     (ua, Fa, ta, ia), (ub, Fb, tb, ib) = res
     assert ia == ib == 21 and np.array_equal(ua, ub)
     assert abs(Fa - Fb) < 1e-12 and abs(ta - tb) < 1e-12 * ta
+
+
+# ---------------------------------------------------------------- FP32 rounding
+@pytest.mark.parametrize("storage,gauge,form,dims,sweeps,F,theta", [
+    (2, 0, 0, (8, 8, 8, 8), 24, 7.257522344783258e-01, 2.701736211561349e-02),
+    (2, 0, 0, (10, 6, 12, 4), 21, 7.276193623189573e-01, 1.633212912676822e-01),
+    (2, 1, 0, (8, 8, 8, 8), 24, 7.625798768001711e-01, 1.400086803561074e-02),
+    (2, 1, 1, (10, 6, 12, 4), 21, 7.610285225105874e-01, 1.163344100478248e-01),
+    (1, 0, 0, (8, 8, 8, 8), 24, 7.257523606919373e-01, 2.701735658892209e-02),
+    (1, 0, 1, (10, 6, 12, 4), 21, 7.261650481157833e-01, 9.432334708808750e-02),
+    (1, 1, 0, (8, 8, 8, 8), 24, 7.625800245700197e-01, 1.400081968762201e-02),
+    (1, 1, 1, (8, 8, 8, 8), 24, 7.627856836447285e-01, 1.110714252386794e-02),
+])
+def test_fp32_rounding_is_pinned(gf, storage, gauge, form, dims, sweeps, F, theta):
+    # F and theta of short FP32 runs as the plain products give them.  Another rounding of the
+    # sweeps moves theta by 1e-7 to 1e-6 of itself and F by 1e-9 and more; the order of the sums
+    # over tiles, the only freedom left, moves them by 2^-44: 1e-10 separates the two.
+    fx = gf.GaugeFixer(dims, gauge, storage)
+    gf.gf_set_overrelax_form(fx.h, form)
+    fx.upload(fields.random_gauge_config(dims, 0.4, 98))
+    r = fx.fix(1e-300, sweeps)
+    fx.close()
+    assert abs(r["F"][0] - F) <= 1e-10 * F and abs(r["theta"][0] - theta) <= 1e-10 * theta
