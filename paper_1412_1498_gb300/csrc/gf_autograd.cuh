@@ -20,8 +20,11 @@
 // same reduction with closed forms for the coefficients), and every power series in X is
 // a polynomial f0 + f1 X + f2 X^2.  Its coefficients come from the scalar recurrence of the
 // powers, X^{n+1} = d_n c0 + (a_n + d_n c1) X + b_n X^2, in place of matrix products: five
-// instructions a term.  Arguments with a spectral radius above 1 are halved first and the
-// polynomial is squared modulo X^3 - c1 X - c0 afterwards.
+// instructions a term.  Arguments with a spectral radius above 1 are halved s times first and the
+// polynomial is squared modulo X^3 - c1 X - c0 afterwards, up to kPolySquarings times: its
+// coefficients grow with the square of the radius where eigenvalues (nearly) coincide, df/dc0
+// faster (gradient off by 1.4e-11 at radius 200).  Above that exp and its derivative are
+// squared as matrices, L -> exp L + L exp, whose errors grow with the radius only.
 //
 // Gradient.  With S = sum_mu W_mu(x) (wF + wT B_mu(x)) + W_mu(x-mu)^+ (wF - wT B_mu(x-mu)),
 // wF = F_bar / (nd Nc V), wT = -4 theta_bar / (Nc V) and B_nu(y) = Delta(y+nu) - Delta(y)
@@ -97,12 +100,20 @@ __device__ __forceinline__ void poly_mul(const c64 (&a)[3], const c64 (&b)[3], d
   out[2] = {gf_fma(c1, p4.re, p2.re), gf_fma(c1, p4.im, p2.im)};
 }
 
-// exp(i 2^s x) = f0 + f1 x + f2 x^2 for the scaled x (x := 2^-s X on return, s the returned
-// value) and, with DERIV, h = df/dc0 at fixed c1 (c0, c1 of the scaled x).
+// Tr X^2 / 2
+__device__ __forceinline__ double herm_c1(const Herm& x) {
+  return 0.5 * gf_fma(x.d0, x.d0, gf_fma(x.d1, x.d1, x.d2 * x.d2)) + (cnorm2(x.x01) + cnorm2(x.x02) + cnorm2(x.x12));
+}
+
+constexpr int kPolySquarings = 3;  // radius 8
+// whether exp_coefficients halves x more often than that
+__device__ __forceinline__ bool exp_is_large(const Herm& x) { return herm_c1(x) * (4.0 / 3.0) > 64.0; }
+
+// exp(i 2^k x) = f0 + f1 x + f2 x^2, k = min(s, kPolySquarings), for the scaled x (x := 2^-s X on
+// return, s the returned value) and, with DERIV, h = df/dc0 at fixed c1 (c0, c1 of the scaled x).
 template <bool DERIV>
 __device__ __forceinline__ int exp_coefficients(Herm& x, c64 (&f)[3], c64 (&h)[3], double& c0, double& c1) {
-  const double n01 = cnorm2(x.x01), n02 = cnorm2(x.x02), n12 = cnorm2(x.x12);
-  c1 = 0.5 * gf_fma(x.d0, x.d0, gf_fma(x.d1, x.d1, x.d2 * x.d2)) + (n01 + n02 + n12);
+  c1 = herm_c1(x);
   // the largest eigenvalue is at most 2 sqrt(c1 / 3)
   int s = 0;
   double r2 = c1 * (4.0 / 3.0);
@@ -171,7 +182,7 @@ __device__ __forceinline__ int exp_coefficients(Herm& x, c64 (&f)[3], c64 (&h)[3
     }
   }
 #pragma unroll 1
-  for (int k = 0; k < s; ++k) {
+  for (int k = 0; k < (s < kPolySquarings ? s : kPolySquarings); ++k) {
     c64 sq[3];
     poly_mul(f, f, c0, c1, sq);
     if (DERIV) {
@@ -189,6 +200,33 @@ __device__ __forceinline__ int exp_coefficients(Herm& x, c64 (&f)[3], c64 (&h)[3
   return s;
 }
 
+__device__ __forceinline__ void m3_mul(const c64* a, const c64* b, c64* out) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      c64 v = cmul_fma(a[3 * i], b[j]);
+      cmac(v, a[3 * i + 1], b[3 + j]);
+      cmac(v, a[3 * i + 2], b[6 + j]);
+      out[3 * i + j] = v;
+    }
+}
+// g -> g^(2^n), and with it the derivative z -> that of the power: the rare sites of large
+// parameters, kept out of the callers' registers
+__device__ __noinline__ void m3_squarings(c64* g, c64* z, int n) {
+#pragma unroll 1
+  for (int k = 0; k < n; ++k) {
+    c64 t[9], u[9];
+    if (z) {
+      m3_mul(g, z, t);
+      m3_mul(z, g, u);
+      for (int e = 0; e < 9; ++e) z[e] = cadd(t[e], u[e]);
+    }
+    m3_mul(g, g, t);
+    for (int e = 0; e < 9; ++e) g[e] = t[e];
+  }
+}
+
 // acc + s a for a real s
 __device__ __forceinline__ void rmac(c64& acc, double s, c64 a) {
   acc.re = gf_fma(s, a.re, acc.re);
@@ -198,6 +236,19 @@ __device__ __forceinline__ void rmac(c64& acc, double s, c64 a) {
 __device__ __forceinline__ void imac(c64& acc, double s, c64 a) {
   acc.re = gf_fma(-s, a.im, acc.re);
   acc.im = gf_fma(s, a.re, acc.im);
+}
+
+// f0 + f1 X + f2 X^2, Q = X^2
+__device__ __forceinline__ void poly_matrix(const c64 (&f)[3], const Herm& X, const Herm& Q, c64* g) {
+  g[0] = f[0]; rmac(g[0], X.d0, f[1]); rmac(g[0], Q.d0, f[2]);
+  g[4] = f[0]; rmac(g[4], X.d1, f[1]); rmac(g[4], Q.d1, f[2]);
+  g[8] = f[0]; rmac(g[8], X.d2, f[1]); rmac(g[8], Q.d2, f[2]);
+  g[1] = cmul_fma(f[1], X.x01); cmac(g[1], f[2], Q.x01);
+  g[2] = cmul_fma(f[1], X.x02); cmac(g[2], f[2], Q.x02);
+  g[5] = cmul_fma(f[1], X.x12); cmac(g[5], f[2], Q.x12);
+  g[3] = cmul_conj_fma(f[1], X.x01); cmac_conj(g[3], f[2], Q.x01);
+  g[6] = cmul_conj_fma(f[1], X.x02); cmac_conj(g[6], f[2], Q.x02);
+  g[7] = cmul_conj_fma(f[1], X.x12); cmac_conj(g[7], f[2], Q.x12);
 }
 
 // ------------------------------------------------------------------------- site and buffers

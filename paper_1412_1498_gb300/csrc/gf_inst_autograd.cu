@@ -13,19 +13,17 @@ __global__ void __launch_bounds__(kT) k_ad_exp(AdArgs a) {
   Herm X = lie_to_X(a.c + 8 * x);
   c64 f[3], h[3];
   double c0, c1;
-  exp_coefficients<false>(X, f, h, c0, c1);
-  const Herm Q = herm_square(X);
+  const int s = exp_coefficients<false>(X, f, h, c0, c1);
   c64 g[9];
-  // g = f0 + f1 X + f2 X^2
-  g[0] = f[0]; rmac(g[0], X.d0, f[1]); rmac(g[0], Q.d0, f[2]);
-  g[4] = f[0]; rmac(g[4], X.d1, f[1]); rmac(g[4], Q.d1, f[2]);
-  g[8] = f[0]; rmac(g[8], X.d2, f[1]); rmac(g[8], Q.d2, f[2]);
-  g[1] = cmul_fma(f[1], X.x01); cmac(g[1], f[2], Q.x01);
-  g[2] = cmul_fma(f[1], X.x02); cmac(g[2], f[2], Q.x02);
-  g[5] = cmul_fma(f[1], X.x12); cmac(g[5], f[2], Q.x12);
-  g[3] = cmul_conj_fma(f[1], X.x01); cmac_conj(g[3], f[2], Q.x01);
-  g[6] = cmul_conj_fma(f[1], X.x02); cmac_conj(g[6], f[2], Q.x02);
-  g[7] = cmul_conj_fma(f[1], X.x12); cmac_conj(g[7], f[2], Q.x12);
+  poly_matrix(f, X, herm_square(X), g);
+  if (s > kPolySquarings) {
+    c64 t[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) t[e] = g[e];
+    m3_squarings(t, nullptr, s - kPolySquarings);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) g[e] = t[e];
+  }
   ad_store9(a.g, a.lat.V, x, g);
 }
 
@@ -125,7 +123,109 @@ __global__ void __launch_bounds__(kT) k_ad_delta(AdArgs a, int t0, int n_t, int 
   }
 }
 
-__global__ void __launch_bounds__(kT) k_ad_backward(AdArgs a, int t0, int n_t) {
+// M = E X + X E and the factors of X^2 and X in the derivative in the direction E (gf_autograd.cuh)
+__device__ __forceinline__ void frechet_terms(const c64 (&E)[9], const Herm& X, const c64 (&h)[3], double c0, double c1,
+                                              c64 (&M)[9], c64& alpha, c64& beta) {
+  const c64 trE = cadd(cadd(E[0], E[4]), E[8]);
+  c64 trEX, trEX2;
+  {
+    const c64 c01 = cconj(X.x01), c02 = cconj(X.x02), c12 = cconj(X.x12);
+    c64 EX[9];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const c64 e0 = E[3 * r], e1 = E[3 * r + 1], e2 = E[3 * r + 2];
+      EX[3 * r] = cmul_fma(e1, c01);
+      cmac(EX[3 * r], e2, c02);
+      rmac(EX[3 * r], X.d0, e0);
+      EX[3 * r + 1] = cmul_fma(e0, X.x01);
+      cmac(EX[3 * r + 1], e2, c12);
+      rmac(EX[3 * r + 1], X.d1, e1);
+      EX[3 * r + 2] = cmul_fma(e0, X.x02);
+      cmac(EX[3 * r + 2], e1, X.x12);
+      rmac(EX[3 * r + 2], X.d2, e2);
+    }
+    trEX = cadd(cadd(EX[0], EX[4]), EX[8]);
+    trEX2 = cmul_fma(EX[1], c01);
+    cmac(trEX2, EX[2], c02);
+    cmac(trEX2, EX[5], c12);
+    cmac(trEX2, EX[3], X.x01);
+    cmac(trEX2, EX[6], X.x02);
+    cmac(trEX2, EX[7], X.x12);
+    rmac(trEX2, X.d0, EX[0]);
+    rmac(trEX2, X.d1, EX[4]);
+    rmac(trEX2, X.d2, EX[8]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const c64 e0 = E[c], e1 = E[3 + c], e2 = E[6 + c];
+      M[c] = EX[c];
+      rmac(M[c], X.d0, e0);
+      cmac(M[c], X.x01, e1);
+      cmac(M[c], X.x02, e2);
+      M[3 + c] = EX[3 + c];
+      cmac(M[3 + c], c01, e0);
+      rmac(M[3 + c], X.d1, e1);
+      cmac(M[3 + c], X.x12, e2);
+      M[6 + c] = EX[6 + c];
+      cmac(M[6 + c], c02, e0);
+      cmac(M[6 + c], c12, e1);
+      rmac(M[6 + c], X.d2, e2);
+    }
+  }
+  alpha = cmul_fma(h[0], trE);
+  beta = cmul_fma(cscale(h[2], c0), trE);
+  cmac(alpha, h[1], trEX);
+  cmac(alpha, h[2], trEX2);
+  cmac(beta, c64{gf_fma(c1, h[2].re, h[0].re), gf_fma(c1, h[2].im, h[0].im)}, trEX);
+  cmac(beta, h[1], trEX2);
+}
+
+// The gradient of a site whose exponential is squared as a matrix: Z, the derivative of exp(i 2^k x)
+// in the direction E, as a whole matrix.  The polynomial's terms leave its multiple of 1 open
+// (they assume a traceless dx), which Tr Z = i 2^k Tr[E exp(i 2^k x)] fixes.  Not inlined: the
+// other sites' registers stay free of it.
+__device__ __noinline__ void ad_gradient_large(const c64* Ep, const double* c, double* out) {
+  c64 E[9], M[9], f[3], h[3], alpha, beta;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) E[e] = Ep[e];
+  Herm X = lie_to_X(c);
+  double c0, c1;
+  const int sh = exp_coefficients<true>(X, f, h, c0, c1);
+  frechet_terms(E, X, h, c0, c1, M, alpha, beta);
+  const Herm Q = herm_square(X);
+  c64 g[9], z[9];
+  poly_matrix(f, X, Q, g);
+  const c64 fz[3] = {{0.0, 0.0}, beta, alpha};
+  poly_matrix(fz, X, Q, z);
+  c64 trEg = {0.0, 0.0}, tr = {0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      cmac(z[3 * i + j], f[1], E[3 * i + j]);
+      cmac(z[3 * i + j], f[2], M[3 * i + j]);
+      cmac(trEg, E[3 * i + j], g[3 * j + i]);
+    }
+  tr = cadd(cadd(z[0], z[4]), z[8]);
+  constexpr double p = 1 << kPolySquarings;
+  const c64 one = {(-p * trEg.im - tr.re) / 3.0, (p * trEg.re - tr.im) / 3.0};
+  z[0] = cadd(z[0], one);
+  z[4] = cadd(z[4], one);
+  z[8] = cadd(z[8], one);
+  m3_squarings(g, z, sh - kPolySquarings);
+  const double s3 = 0.57735026918962576451;
+  const double sc = __hiloint2double((1023 - sh) << 20, 0);  // 2^-s: dx = 2^-s dX
+  // Re Tr[lambda_a Z]
+  out[0] = sc * (z[1].re + z[3].re);
+  out[1] = sc * (z[3].im - z[1].im);
+  out[2] = sc * (z[0].re - z[4].re);
+  out[3] = sc * (z[2].re + z[6].re);
+  out[4] = sc * (z[6].im - z[2].im);
+  out[5] = sc * (z[5].re + z[7].re);
+  out[6] = sc * (z[7].im - z[5].im);
+  out[7] = sc * (s3 * (z[0].re + z[4].re - 2.0 * z[8].re));
+}
+
+__global__ void __launch_bounds__(kT, 4) k_ad_backward(AdArgs a, int t0, int n_t) {
   const unsigned i = blockIdx.x * (unsigned)kT + threadIdx.x;
   if (i >= 2u * (unsigned)a.lat.V3h * (unsigned)n_t) return;
   const AdSite s = ad_site(a.lat, i, t0);
@@ -178,61 +278,18 @@ __global__ void __launch_bounds__(kT) k_ad_backward(AdArgs a, int t0, int n_t) {
     }
   }
   Herm X = lie_to_X(a.c + 8 * x);
+  if (exp_is_large(X)) {
+    c64 t[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) t[e] = E[e];
+    ad_gradient_large(t, a.c + 8 * x, a.grad + 8 * x);
+    return;
+  }
   c64 f[3], h[3];
   double c0, c1;
   const int sh = exp_coefficients<true>(X, f, h, c0, c1);
-  // EX, and M = EX + XE
-  c64 M[9];
-  const c64 trE = cadd(cadd(E[0], E[4]), E[8]);
-  c64 trEX, trEX2;
-  {
-    const c64 c01 = cconj(X.x01), c02 = cconj(X.x02), c12 = cconj(X.x12);
-    c64 EX[9];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const c64 e0 = E[3 * r], e1 = E[3 * r + 1], e2 = E[3 * r + 2];
-      EX[3 * r] = cmul_fma(e1, c01);
-      cmac(EX[3 * r], e2, c02);
-      rmac(EX[3 * r], X.d0, e0);
-      EX[3 * r + 1] = cmul_fma(e0, X.x01);
-      cmac(EX[3 * r + 1], e2, c12);
-      rmac(EX[3 * r + 1], X.d1, e1);
-      EX[3 * r + 2] = cmul_fma(e0, X.x02);
-      cmac(EX[3 * r + 2], e1, X.x12);
-      rmac(EX[3 * r + 2], X.d2, e2);
-    }
-    trEX = cadd(cadd(EX[0], EX[4]), EX[8]);
-    trEX2 = cmul_fma(EX[1], c01);
-    cmac(trEX2, EX[2], c02);
-    cmac(trEX2, EX[5], c12);
-    cmac(trEX2, EX[3], X.x01);
-    cmac(trEX2, EX[6], X.x02);
-    cmac(trEX2, EX[7], X.x12);
-    rmac(trEX2, X.d0, EX[0]);
-    rmac(trEX2, X.d1, EX[4]);
-    rmac(trEX2, X.d2, EX[8]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const c64 e0 = E[c], e1 = E[3 + c], e2 = E[6 + c];
-      M[c] = EX[c];
-      rmac(M[c], X.d0, e0);
-      cmac(M[c], X.x01, e1);
-      cmac(M[c], X.x02, e2);
-      M[3 + c] = EX[3 + c];
-      cmac(M[3 + c], c01, e0);
-      rmac(M[3 + c], X.d1, e1);
-      cmac(M[3 + c], X.x12, e2);
-      M[6 + c] = EX[6 + c];
-      cmac(M[6 + c], c02, e0);
-      cmac(M[6 + c], c12, e1);
-      rmac(M[6 + c], X.d2, e2);
-    }
-  }
-  c64 alpha = cmul_fma(h[0], trE), beta = cmul_fma(cscale(h[2], c0), trE);
-  cmac(alpha, h[1], trEX);
-  cmac(alpha, h[2], trEX2);
-  cmac(beta, c64{gf_fma(c1, h[2].re, h[0].re), gf_fma(c1, h[2].im, h[0].im)}, trEX);
-  cmac(beta, h[1], trEX2);
+  c64 M[9], alpha, beta;
+  frechet_terms(E, X, h, c0, c1, M, alpha, beta);
   // Z = f1 E + f2 M + alpha X^2 + beta X; only its Hermitian part counts.  The X terms have
   // a Hermitian part Re(alpha) X^2 + Re(beta) X.
   const Herm Q = herm_square(X);

@@ -157,3 +157,57 @@ def test_slabs_equal_the_whole(gf, gauge):
     (F0, t0, g0), (F1, t1, g1) = res
     assert abs(F1 - F0) < 1e-12 * abs(F0) + 1e-15 and abs(t1 - t0) < 1e-12 * t0
     assert float((g1 - g0.repeat(*reps[::-1], 1)).abs().max()) < 1e-12 * float(g0.abs().max())
+
+
+def _exp_frechet(X, E=None):
+    # exp(iX) of Hermitian X and the derivative of exp(i .) in the direction E, from the
+    # eigenvalues (Daleckii-Krein; the divided differences i exp(i (a + b) / 2) sinc((a - b) / 2) have
+    # no cancellation): errors of a rounding times the spectral radius
+    lam, V = np.linalg.eigh(X)
+    Vh = V.conj().swapaxes(-1, -2)
+    if E is None:
+        return (V * np.exp(1j * lam)[..., None, :]) @ Vh
+    a, b = lam[..., :, None], lam[..., None, :]
+    phi = 1j * np.exp(0.5j * (a + b)) * np.sinc((a - b) / (2 * np.pi))
+    return V @ ((Vh @ E @ V) * phi) @ Vh
+
+
+@pytest.mark.parametrize("along", ["lambda_8", "nearly", "random"])
+@pytest.mark.parametrize("radius", [0.3, 3.0, 7.5, 20.0, 200.0, 2000.0])
+def test_gradient_at_large_parameters(gf, radius, along):
+    # zero to eleven squarings of the exponential, with equal, nearly equal and other eigenvalues.
+    # Squaring a unitary matrix doubles its relative error, which after log2(radius) squarings is
+    # radius * 2^-52 times a few operations' errors on either side: 50 radius 2^-52 (radius >= 4)
+    from paper_1412_1498_gb300.autograd import functional_theta
+    dims = (2, 2, 4, 2)
+    lat = dims[::-1]
+    rng = np.random.default_rng(8)
+    c = rng.normal(size=lat + (8,))
+    if along != "random":
+        c[..., :7] *= 0.0 if along == "lambda_8" else 1e-7
+        c[..., 7] = np.where(c[..., 7] < 0, -1.0, 1.0) * (0.5 + 0.5 * rng.random(lat))
+    X = np.einsum("...a,aij->...ij", c, fields.gell_mann())
+    scale = radius / np.abs(np.linalg.eigvalsh(X)).max()
+    c, X = c * scale, X * scale
+    U = fields.random_gauge_config(dims, 0.5, 7)
+    g = torch.from_numpy(_exp_frechet(X)).requires_grad_(True)
+    Ut = torch.from_numpy(U)
+    step = lambda f, mu, n: torch.roll(f, -n, dims=3 - mu)
+    W = [g @ Ut[..., mu, :, :] @ step(g, mu, 1).mH for mu in range(4)]
+    D = sum(step(w, mu, -1) - w for mu, w in enumerate(W))
+    D = D - D.mH
+    D = D - D.diagonal(dim1=-2, dim2=-1).sum(-1)[..., None, None] / 3 * torch.eye(3)
+    n = float(np.prod(dims))
+    F = sum(w.diagonal(dim1=-2, dim2=-1).real.sum() for w in W) / (12 * n)
+    th = (D.abs() ** 2).sum() / (3 * n)
+    (G,) = torch.autograd.grad(0.3 * th - F, g)      # dL = Re sum conj(G) dg = Re Tr[E dg]
+    L = _exp_frechet(X, G.numpy().conj().swapaxes(-1, -2))
+    want = np.einsum("aij,...ji->...a", fields.gell_mann(), L).real.reshape(-1, 8)
+    fx = make(gf, dims, 0, U)
+    p = torch.from_numpy(c.reshape(-1, 8)).cuda().requires_grad_(True)
+    Fg, tg = functional_theta(p, fx)
+    (got,) = torch.autograd.grad(0.3 * tg - Fg, p)
+    fx.close()
+    tol = 50 * max(radius, 4.0) * 2.0 ** -52
+    assert abs(Fg.item() - F.item()) < tol and abs(tg.item() - th.item()) < tol * th.item()
+    assert np.abs(got.cpu().numpy() - want).max() < tol * np.abs(want).max()
