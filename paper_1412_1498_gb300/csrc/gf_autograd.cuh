@@ -312,6 +312,24 @@ __device__ __forceinline__ void ad_store9(c64* base, long long n, long long at, 
   for (int e = 0; e < 9; ++e) p[e * n] = make_double2(m[e].re, m[e].im);
 }
 
+__device__ __forceinline__ int ad_storage_idx(const LatDev& lat, const AdSite& s) {
+  return ((s.x + s.y + s.z + s.t) & 1) * lat.Vh + (int)(ad_lexi(lat, s) >> 1);
+}
+// W_mu(s) from the buffer, or formed (BUF false)
+template <bool BUF>
+__device__ __forceinline__ void ad_link(const AdArgs& a, const AdSite& s, int mu, c64 (&u)[9]) {
+  if constexpr (BUF) {
+    ad_load9(a.w + 9 * mu * a.w_n, a.w_n, ad_wplace(a, s), u);
+  } else {
+    c64 g[9];
+    Store<GF_FP64_18>::load(a.links + a.lat.off_bytes, a.lat.V, mu, ad_storage_idx(a.lat, s), u);
+    ad_load9(a.g, a.lat.V, ad_lexi(a.lat, s), g);
+    left_mul(g, u);
+    ad_load9(a.g, a.lat.V, ad_lexi(a.lat, ad_step(a.lat, s, mu, +1)), g);
+    right_mul_dag(u, g);
+  }
+}
+
 // anti-Hermitian traceless matrix: upper triangle and the imaginary diagonal
 struct AntiH {
   c64 b01, b02, b12;

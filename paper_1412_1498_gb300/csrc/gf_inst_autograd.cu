@@ -29,7 +29,8 @@ __global__ void __launch_bounds__(kT) k_ad_exp(AdArgs a) {
 
 // W_mu(x) = g(x) U_mu(x) g(x+mu)^+ for the sites of `n_t` slices from a.w_t0 on, and Re Tr
 // of those whose slice is one of the n_f from f_t0 on (a slab's halo slice belongs to
-// another slab's F).
+// another slab's F).  Without a buffer (BUF false): the whole lattice, for F alone.
+template <bool BUF>
 __global__ void __launch_bounds__(kT) k_ad_links(AdArgs a, int n_t, int f_t0, int n_f, int part0) {
   __shared__ double red[32];
   const unsigned i = blockIdx.x * (unsigned)kT + threadIdx.x;
@@ -37,8 +38,8 @@ __global__ void __launch_bounds__(kT) k_ad_links(AdArgs a, int n_t, int f_t0, in
   double v[1] = {0.0};
   if (i < n) {
     const AdSite s = ad_site(a.lat, i, a.w_t0);
-    const long long lexi = ad_lexi(a.lat, s), place = ad_wplace(a, s);
-    const int idx = ((s.x + s.y + s.z + s.t) & 1) * a.lat.Vh + (int)(lexi >> 1);
+    const long long lexi = ad_lexi(a.lat, s), place = BUF ? ad_wplace(a, s) : 0;
+    const int idx = ad_storage_idx(a.lat, s);
     int tf = s.t - f_t0;
     if (tf < 0) tf += a.lat.L[3];
     c64 g[9];
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(kT) k_ad_links(AdArgs a, int n_t, int f_t0, in
       left_mul(g, u);
       right_mul_dag(u, gn);
       f += u[0].re + u[4].re + u[8].re;
-      ad_store9(a.w + 9 * mu * a.w_n, a.w_n, place, u);
+      if constexpr (BUF) ad_store9(a.w + 9 * mu * a.w_n, a.w_n, place, u);
     }
     if (tf < n_f) v[0] = f;
   }
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(kT) k_ad_links(AdArgs a, int n_t, int f_t0, in
 
 // Delta(x) (Eq. (3)) of the slices t0 .. t0 + n_t - 1 and Tr[Delta Delta^+].  The last block
 // of the last slab's launch adds the partials of all `n_parts` blocks in a fixed order.
+template <bool BUF>
 __global__ void __launch_bounds__(kT) k_ad_delta(AdArgs a, int t0, int n_t, int part0, int n_links_parts,
                                                  int n_parts) {
   __shared__ double red[64];
@@ -75,13 +77,11 @@ __global__ void __launch_bounds__(kT) k_ad_delta(AdArgs a, int t0, int n_t, int 
     // D = A - A^+, A = sum_nu W_nu(x - nu) - W_nu(x): upper elements, imaginary diagonal
     c64 d01 = {0.0, 0.0}, d02 = d01, d12 = d01;
     double e0 = 0.0, e1 = 0.0, e2 = 0.0;
-    const long long at = ad_wplace(a, s);
 #pragma unroll 1
     for (int nu = 0; nu < a.nd; ++nu) {
       c64 f[9], b[9];
-      const c64* w = a.w + 9 * nu * a.w_n;
-      ad_load9(w, a.w_n, at, f);
-      ad_load9(w, a.w_n, ad_wplace(a, ad_step(a.lat, s, nu, -1)), b);
+      ad_link<BUF>(a, s, nu, f);
+      ad_link<BUF>(a, ad_step(a.lat, s, nu, -1), nu, b);
       d01 = cadd(d01, csub(csub(b[1], f[1]), cconj(csub(b[3], f[3]))));
       d02 = cadd(d02, csub(csub(b[2], f[2]), cconj(csub(b[6], f[6]))));
       d12 = cadd(d12, csub(csub(b[5], f[5]), cconj(csub(b[7], f[7]))));
@@ -225,11 +225,12 @@ __device__ __noinline__ void ad_gradient_large(const c64* Ep, const double* c, d
   out[7] = sc * (s3 * (z[0].re + z[4].re - 2.0 * z[8].re));
 }
 
+template <bool BUF>
 __global__ void __launch_bounds__(kT, 4) k_ad_backward(AdArgs a, int t0, int n_t) {
   const unsigned i = blockIdx.x * (unsigned)kT + threadIdx.x;
   if (i >= 2u * (unsigned)a.lat.V3h * (unsigned)n_t) return;
   const AdSite s = ad_site(a.lat, i, t0);
-  const long long x = ad_lexi(a.lat, s), at = ad_wplace(a, s);
+  const long long x = ad_lexi(a.lat, s);
   const double V = (double)a.lat.V;
   const double wF = a.upstream[0] / ((double)a.nd * 3.0 * V);
   const double wT = -a.upstream[1] * 4.0 / (3.0 * V);
@@ -239,11 +240,10 @@ __global__ void __launch_bounds__(kT, 4) k_ad_backward(AdArgs a, int t0, int n_t
 #pragma unroll 1
   for (int mu = 0; mu < a.nd; ++mu) {
     const AdSite sp = ad_step(a.lat, s, mu, +1), sm = ad_step(a.lat, s, mu, -1);
-    const c64* w = a.w + 9 * mu * a.w_n;
     c64 u[9];
-    ad_load9(w, a.w_n, at, u);
+    ad_link<BUF>(a, s, mu, u);
     add_antih_product<false>(R, u, antih_sub(ad_load_delta(a, ad_lexi(a.lat, sp)), D));
-    ad_load9(w, a.w_n, ad_wplace(a, sm), u);
+    ad_link<BUF>(a, sm, mu, u);
     // -B_mu(x-mu) = Delta(x-mu) - Delta(x)
     add_antih_product<true>(R, u, antih_sub(ad_load_delta(a, ad_lexi(a.lat, sm)), D));
   }
@@ -326,25 +326,31 @@ static unsigned int blocks(long long n) { return (unsigned int)((n + kT - 1) / k
 
 // Time slices of sites that one pass over the W buffer serves: all of them when the buffer
 // holds the lattice, else as many as it holds besides the slice before them (whose time
-// links they need).
-static int slab_slices(const AdArgs& a) { return a.w_slices >= a.lat.L[3] ? a.lat.L[3] : a.w_slices - 1; }
+// links they need).  Without a buffer (w_slices = 0) one pass serves the lattice.
+static int slab_slices(int w_slices, int Lt) { return w_slices == 0 || w_slices >= Lt ? Lt : w_slices - 1; }
+static int slab_slices(const AdArgs& a) { return slab_slices(a.w_slices, a.lat.L[3]); }
 
 // Slices of W the workspace keeps: the whole lattice up to kWBytes (15 million sites), else
 // what kWBytes hold (at least two slices); larger lattices are served in slabs, which
-// form the links twice in the backward.
+// form the links twice in the backward.  With few and very large time slices two of them
+// can cost far more than the lattice's other buffers (32 x 32 x 65536 sites: 77 GB); a lattice on which the
+// buffer would take more than kWBytes above the 80 bytes a site that it saves in g and Delta
+// keeps none (0), and its passes form the links they need (twice as many products).
 int ad_w_slices(const int* L) {
   constexpr size_t kWBytes = (size_t)8 << 30;
-  const size_t slice = (size_t)L[0] * L[1] * L[2] * 4 * 9 * 16;
+  const size_t sites = (size_t)L[0] * L[1] * L[2], slice = sites * 4 * 9 * 16;
   const size_t k = kWBytes / slice;
-  return k >= (size_t)L[3] ? L[3] : (k < 2 ? 2 : (int)k);
+  if (k >= (size_t)L[3]) return L[3];
+  if (k >= 2) return (int)k;
+  return 2 * slice <= kWBytes + 80 * sites * L[3] ? 2 : 0;
 }
 
 size_t ad_partial_doubles(const int* L) {
   // one pair per block, slabs of at least one slice each with one halo slice
   const long long V3 = (long long)L[0] * L[1] * L[2];
-  const int w = ad_w_slices(L), n = w >= L[3] ? L[3] : w - 1;
+  const int w = ad_w_slices(L), n = slab_slices(w, L[3]);
   const int slabs = (L[3] + n - 1) / n;
-  return 2 * (size_t)slabs * (size_t)((V3 * w + kT - 1) / kT);
+  return 2 * (size_t)slabs * (size_t)((V3 * (w == 0 ? L[3] : w) + kT - 1) / kT);
 }
 
 // Runs `use(t0, n, part)` for each slab with its links in the W buffer.
@@ -358,7 +364,8 @@ static void for_slabs(AdArgs& a, cudaStream_t s, int* link_parts, F use) {
     const int nt = m == Lt ? Lt : m + 1;
     a.w_t0 = nt == Lt ? 0 : (t0 + Lt - 1) % Lt;
     const unsigned nb = blocks(V3 * nt);
-    k_ad_links<<<nb, kT, 0, s>>>(a, nt, t0, m, lp);
+    if (a.w_slices) k_ad_links<true><<<nb, kT, 0, s>>>(a, nt, t0, m, lp);
+    else k_ad_links<false><<<nb, kT, 0, s>>>(a, nt, t0, m, lp);
     lp += (int)nb;
     use(t0, m);
   }
@@ -378,7 +385,8 @@ static void delta_pass(AdArgs& a, cudaStream_t s) {
   int lp = 0, dp = 0;
   for_slabs(a, s, &lp, [&](int t0, int m) {
     const unsigned nb = blocks(V3 * m);
-    k_ad_delta<<<nb, kT, 0, s>>>(a, t0, m, dp, n_lp, n_dp);
+    if (a.w_slices) k_ad_delta<true><<<nb, kT, 0, s>>>(a, t0, m, dp, n_lp, n_dp);
+    else k_ad_delta<false><<<nb, kT, 0, s>>>(a, t0, m, dp, n_lp, n_dp);
     dp += (int)nb;
   });
 }
@@ -394,12 +402,17 @@ void launch_ad_backward(const AdArgs& args, cudaStream_t s) {
   k_ad_exp<<<blocks(a.lat.V), kT, 0, s>>>(a);
   delta_pass(a, s);
   const long long V3 = 2LL * a.lat.V3h;
-  if (slab_slices(a) >= a.lat.L[3]) {  // W of the whole lattice is still there
-    k_ad_backward<<<blocks(V3 * a.lat.L[3]), kT, 0, s>>>(a, 0, a.lat.L[3]);
+  const int Lt = a.lat.L[3];
+  if (a.w_slices == 0) {
+    k_ad_backward<false><<<blocks(V3 * Lt), kT, 0, s>>>(a, 0, Lt);
+    return;
+  }
+  if (slab_slices(a) >= Lt) {  // W of the whole lattice is still there
+    k_ad_backward<true><<<blocks(V3 * Lt), kT, 0, s>>>(a, 0, Lt);
     return;
   }
   int lp = 0;
-  for_slabs(a, s, &lp, [&](int t0, int m) { k_ad_backward<<<blocks(V3 * m), kT, 0, s>>>(a, t0, m); });
+  for_slabs(a, s, &lp, [&](int t0, int m) { k_ad_backward<true><<<blocks(V3 * m), kT, 0, s>>>(a, t0, m); });
 }
 
 }  // namespace gf

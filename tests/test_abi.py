@@ -142,3 +142,16 @@ def test_noalloc_rejects_wrapping_or_oversized_volume_on_the_host(dims):
         gf.gf_functional_theta_noalloc(dims, gf.GF_LANDAU, 256, 512)
     assert e.value.code == gf.GF_EINVAL
     assert "too large" in gf.gf_last_error(None)
+
+
+@pytest.mark.parametrize("dims", [(32, 32, 65536, 4), (250, 250, 250, 2), (250, 250, 250, 16), (208, 208, 208, 2), (64, 64, 64, 128),
+                                  (32, 32, 32, 32)])
+def test_autograd_scratch_is_bounded(dims):
+    # g and Delta (208 bytes a site) and a link buffer of 8 GiB at most above the 288 bytes a site of
+    # kernels that keep whole matrices: large time slices do not make a lattice too big for the GPU
+    V = 1
+    for n in dims:
+        V *= n
+    extra = (gf.gf_workspace_bytes([dims], gf.GF_LANDAU, gf.GF_FP64_18, gf.GF_FLAG_AUTOGRAD)
+             - gf.gf_workspace_bytes([dims], gf.GF_LANDAU, gf.GF_FP64_18))
+    assert 208 * V <= extra <= 288 * V + 2 ** 33 + V // 4 + 2 ** 20

@@ -211,3 +211,26 @@ def test_gradient_at_large_parameters(gf, radius, along):
     tol = 50 * max(radius, 4.0) * 2.0 ** -52
     assert abs(Fg.item() - F.item()) < tol and abs(tg.item() - th.item()) < tol * th.item()
     assert np.abs(got.cpu().numpy() - want).max() < tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("gauge", [0, 1])
+def test_without_a_link_buffer_equals_the_small_field(gf, gauge):
+    # two time slices of 208^3 sites: no link buffer (see test_slabs_equal_the_whole for the rest)
+    from paper_1412_1498_gb300.autograd import functional_theta
+    small, n = (8, 8, 8, 2), 26
+    big = tuple(n * v for v in small[:3]) + (2,)
+    U = torch.from_numpy(fields.random_gauge_config(small, 0.5, 104)).cuda()
+    c = torch.from_numpy(np.random.default_rng(5).normal(scale=0.3, size=small[::-1] + (8,))).cuda()
+    res = []
+    for dims, r in ((small, 1), (big, n)):
+        fx = gf.GaugeFixer(dims, gauge, gf.GF_FP64_18, autograd=True)
+        fx.upload(U.repeat(1, r, r, r, 1, 1, 1))
+        p = c.repeat(1, r, r, r, 1).reshape(-1, 8).contiguous().requires_grad_(True)
+        F, th = functional_theta(p, fx)
+        (g,) = torch.autograd.grad(0.3 * th - F, p)
+        res.append((F.item(), th.item(), g.reshape(dims[::-1] + (8,)) * float(r) ** 3))
+        fx.close()
+        del fx, p
+    (F0, t0, g0), (F1, t1, g1) = res
+    assert abs(F1 - F0) < 1e-12 * abs(F0) + 1e-15 and abs(t1 - t0) < 1e-12 * t0
+    assert float((g1 - g0.repeat(1, n, n, n, 1)).abs().max()) < 1e-12 * float(g0.abs().max())
