@@ -257,18 +257,23 @@ GF_API int gf_set_reproducible(gf_handle *h, int on);         /* [0]; 1 = FP64-1
                                   fused multiply-add and with IEEE divisions, in the
                                   oracle's operation order (bit-reproducible results);
                                   no effect on the other storages */
-GF_API int gf_set_block_size(gf_handle *h, int threads);      /* [128]; 64, 128 or 256; no effect
-                                  on FP64 storages (one-warp blocks) and on single lattices of
-                                  up to 2^14 sites (a warp per direction) */
+GF_API int gf_set_block_size(gf_handle *h, int threads);      /* [128]; 64, 128 or 256.  128 leaves
+                                  the choice to the library (see the sweep kernels below); 64 and
+                                  256 are taken as they are */
 
 /* Half-sweep kernel for FP32-12 storage: GF_SWEEP_REGISTER holds each site's 8 links in
    registers; GF_SWEEP_PIPELINED stages them through shared memory with asynchronous
    copies one tile ahead (persistent CTAs).  Both give the same results.  AUTO [default]
-   = PIPELINED for FP32-12, except that a single lattice of up to 2^14 sites takes the
-   direction-per-warp kernel (which also sweeps FP32-18 and FP64-18 lattices of that size)
-   and gf_fix runs the loop of several units on up to 2^17 sites in one cooperative kernel;
-   the links are the same bits.  Other storages always use the register kernel, and asking
-   them for PIPELINED returns GF_EINVAL. */
+   = PIPELINED for FP32-12.  Other storages have the register kernel only (AUTO and REGISTER
+   are the same), and asking them for PIPELINED returns GF_EINVAL.
+   With the default block size, and unless REGISTER is asked of an FP32-12 handle, the library
+   takes other kernels for
+   - one FP32-12 or FP32-18 lattice with one convergence unit, and FP64-18 lattices, of up to
+     2^14 sites in all: a warp per direction;
+   - FP64 storages above that: blocks of one warp;
+   - gf_fix of several units on up to 2^17 sites in FP32-12 or FP32-18 (first-order form, no
+     history, at most 128 units, not mixed): the loop in one cooperative kernel.
+   The links are the same bits with every choice. */
 /* Arithmetic of the polish phase of a mixed-precision gf_fix (GF_FLAG_MIXED):
    GF_POLISH_SPLIT [default]: double-float sweeps (each real an unevaluated sum of two
    floats, about 48-bit precision, no FP64 arithmetic in the sweep) with the first-order

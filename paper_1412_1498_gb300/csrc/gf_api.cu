@@ -123,6 +123,7 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr size_t kStagingMax = 32u << 20;  // bytes of canonical links per host copy
 constexpr int kMinTile = 32;
+constexpr int kDefaultThreads = 128;
 constexpr int kGraphSweeps = 16;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -313,7 +314,7 @@ struct gf_handle {
   // host copies
   std::vector<LatDev> lats, lats64;
   int n_tiles = 0, n_units = 0;
-  int threads = 128;  // block size set by the caller
+  int threads = kDefaultThreads;  // block size set by the caller
   int tile = 128;     // sites per tile = threads of a sweep block (tile_sites_of)
   // settings
   double omega = 1.7, eps_switch = 1e-8;
@@ -395,24 +396,35 @@ char* cur_links(const gf_handle* h) { return h->cur >= 1 ? h->links64 : h->links
 LatDev* cur_lats(const gf_handle* h) { return h->cur >= 1 ? h->d_lats64 : h->d_lats; }
 const LatDev& cur_lat_host(const gf_handle* h, int l) { return h->cur >= 1 ? h->lats64[l] : h->lats[l]; }
 
+// Whether the settings leave the kernel to the library: the default block size, and for FP32-12
+// not the register kernel (PIPELINED is what AUTO means there; the other storages have no second
+// kernel to ask for).
+bool library_chooses(const gf_handle* h) {
+  return h->threads == kDefaultThreads && !(h->storage == GF_FP32_12 && h->variant == GF_SWEEP_REGISTER);
+}
+
 // Whether the handle's sweeps take the direction-per-warp kernel (gf_sweep_dir.cuh, which says
 // where the line lies).  FP32 handles with many units have their loop in one kernel instead.
 constexpr long long kDirSites = 1LL << 14;
 bool dir_kernel_serves(const gf_handle* h) {
+  if (!library_chooses(h)) return false;
   long long sites = 0;
   for (const LatDev& lat : h->lats) sites += lat.V;
   if (sites > kDirSites) return false;
   if (h->storage == GF_FP64_18) return true;
-  return h->n_units == 1 && (h->storage == GF_FP32_18 || (h->storage == GF_FP32_12 && h->variant == GF_SWEEP_AUTO));
+  return h->n_units == 1 && (h->storage == GF_FP32_18 || h->storage == GF_FP32_12);
 }
 
-// Sites per tile.  FP64 storages take one warp: their sweeps are bound by the FP64 pipe, so
+// Sites per tile: the block size of the settings when it is not the default.  By default FP64
+// storages take one warp: their sweeps are bound by the FP64 pipe, so
 // what counts is that every SM gets the same number of warps (some ten fit
-// whatever the block size).  16^4 half-sweep 97 -> 87 us against blocks of
-// 128 sites (256 blocks, two on some SMs and one on others); 8^4 about three times faster.
+// whatever the block size).  us a sweep, tiles of 128 sites -> 32, for FP64-18, FP64-12, FP64-8:
+// 16^4 (256 blocks of 128, two on some SMs and one on others) 187 -> 173, 198 -> 178, 564 -> 499;
+// 20x12x18x10 188 -> 155, 199 -> 154, 565 -> 398; 8^4 FP64-12 105 -> 98, FP64-8 297 -> 271; 24^4
+// 798 -> 803, 850 -> 856, 2510 -> 2516.
 // So do the lattices of the direction-per-warp kernel, whose blocks work on 32 sites.
-// Other handles take the block size of the settings.
 int tile_sites_of(const gf_handle* h) {
+  if (h->threads != kDefaultThreads) return h->threads;
   return is_fp64_storage(h->storage) || dir_kernel_serves(h) ? kMinTile : h->threads;
 }
 
@@ -761,7 +773,7 @@ int run_phase(gf_handle* h, double eps, int budget, int* done) {
 bool loop_kernel_serves(const gf_handle* h) {
   if (h->cur != 0 || (h->storage != GF_FP32_12 && h->storage != GF_FP32_18)) return false;
   if (h->form != GF_OR_FIRST_ORDER) return false;
-  if (h->variant != GF_SWEEP_AUTO || h->tile != kLoopThreads || h->hist || h->n_units == 1 || h->n_units > kLoopUnits) return false;
+  if (!library_chooses(h) || h->tile != kLoopThreads || h->hist || h->n_units == 1 || h->n_units > kLoopUnits) return false;
   long long sites = 0;
   for (const LatDev& lat : h->lats) sites += lat.V;
   return sites <= kLoopSites && h->n_tiles <= 4 * (kLoopSites / 2 / kLoopThreads);

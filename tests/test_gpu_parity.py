@@ -650,3 +650,30 @@ def test_fp32_rounding_is_pinned(gf, storage, gauge, form, dims, sweeps, F, thet
     r = fx.fix(1e-300, sweeps)
     fx.close()
     assert abs(r["F"][0] - F) <= 1e-10 * F and abs(r["theta"][0] - theta) <= 1e-10 * theta
+
+
+# ---------------------------------------------------------------- settings of small handles
+@pytest.mark.parametrize("storage", [0, 1, 2])
+def test_block_size_reaches_small_lattices(gf, storage):
+    # every block size is taken, on FP64 storage and on lattices of the direction-per-warp kernel
+    # too: other tiles, so F is summed in another order; the links are the same bits.  FP64-18 in
+    # blocks of 256 (one thread a site, 12 blocks for 152 SMs) takes over three times the default's time.
+    import time
+    dims = (8, 8, 8, 6)
+    U = fields.random_gauge_config(dims, 0.4, 94)
+    out, ts = [], {}
+    for threads in (128, 64, 256):
+        fx = gf.GaugeFixer(dims, gf.GF_LANDAU, storage)
+        gf.gf_set_block_size(fx.h, threads)
+        fx.upload(U)
+        r = fx.fix(1e-300, 23)
+        out.append((fx.download(), r["F"][0], r["theta"][0]))
+        ts[threads] = []
+        for _ in range(4):
+            t0 = time.perf_counter()
+            fx.fix(1e-300, 100)
+            ts[threads].append(time.perf_counter() - t0)
+        fx.close()
+    assert storage != gf.GF_FP64_18 or min(ts[256]) > 1.5 * min(ts[128])
+    for u, F, th in out[1:]:
+        assert np.array_equal(u, out[0][0]) and abs(F - out[0][1]) < 1e-12 and abs(th - out[0][2]) < 1e-12 * th
