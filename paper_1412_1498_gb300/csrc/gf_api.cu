@@ -1773,13 +1773,27 @@ int gf_autotune(gf_handle* h, int* threads_out, int* variant_out) {
   // gauge-invariant content is unchanged), but a run meant to start from the original
   // configuration uploads it again afterwards.
   const int st = cur_storage(h);
+  // A handle whose gf_fix loop is one kernel under the default settings keeps them: no kernel
+  // of separate launches comes near it (gf_loop.cuh).
+  {
+    const int threads = h->threads, variant = h->variant;
+    h->variant = st == GF_FP32_12 ? GF_SWEEP_PIPELINED : GF_SWEEP_REGISTER;
+    int rc = gf_set_block_size(h, kDefaultThreads);
+    if (rc != GF_OK) return rc;
+    if (loop_kernel_serves(h) && !(h->flags & GF_FLAG_MIXED)) {
+      drop_graphs(h);
+      if (threads_out) *threads_out = h->threads;
+      if (variant_out) *variant_out = h->variant;
+      return GF_OK;
+    }
+    h->variant = variant;
+    if ((rc = gf_set_block_size(h, threads)) != GF_OK) return rc;
+  }
   std::vector<std::pair<int, int>> cands;
   for (int t : {64, 128, 256}) {
     cands.push_back({t, GF_SWEEP_REGISTER});
     if (st == GF_FP32_12) cands.push_back({t, GF_SWEEP_PIPELINED});
   }
-  // what AUTO takes on a small lattice; reported as PIPELINED, AUTO's meaning
-  if (st == GF_FP32_12 && h->tile == kMinTile) cands.push_back({128, GF_SWEEP_AUTO});
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
@@ -1815,7 +1829,7 @@ int gf_autotune(gf_handle* h, int* threads_out, int* variant_out) {
   drop_graphs(h);
   if ((rc = gf_set_block_size(h, bt)) != GF_OK) return rc;
   if (threads_out) *threads_out = bt;
-  if (variant_out) *variant_out = bv == GF_SWEEP_AUTO && h->storage == GF_FP32_12 ? GF_SWEEP_PIPELINED : bv;
+  if (variant_out) *variant_out = bv;
   return GF_OK;
 }
 

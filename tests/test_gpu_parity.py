@@ -652,7 +652,36 @@ def test_fp32_rounding_is_pinned(gf, storage, gauge, form, dims, sweeps, F, thet
     assert abs(r["F"][0] - F) <= 1e-10 * F and abs(r["theta"][0] - theta) <= 1e-10 * theta
 
 
-# ---------------------------------------------------------------- settings of small handles
+# ---------------------------------------------------------------- autotuner and small handles
+@pytest.mark.parametrize("storage", [1, 2])
+def test_tuned_small_handle_keeps_its_loop(gf, storage):
+    # 12^3 x 16 Coulomb: gf_fix's one-kernel loop takes about 2/3 of the launched loop's time (17 to 20
+    # launches' worth a sweep); a tuned handle, and one with the tuned pair set, must keep it.
+    # Best of five calls of 200 sweeps each; 1.15 lies halfway between the same and the launched loop.
+    import time
+    dims = (12, 12, 12, 16)
+    U = torch.from_numpy(fields.random_gauge_config(dims, 0.4, 99)).cuda()
+
+    def best(fx):
+        ts = []
+        for _ in range(6):
+            fx.upload(U)
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            fx.fix(1e-300, 200)
+            ts.append(time.perf_counter() - t0)
+        return min(ts)
+    plain, tuned, other = (gf.GaugeFixer(dims, gf.GF_COULOMB, storage) for _ in range(3))
+    tuned.upload(U)
+    pair = gf.gf_autotune(tuned.h)
+    gf.gf_set_block_size(other.h, pair[0])
+    gf.gf_set_sweep_variant(other.h, pair[1])
+    t = [best(fx) for fx in (plain, tuned, other)]
+    for fx in (plain, tuned, other):
+        fx.close()
+    assert t[1] < 1.15 * t[0] and t[2] < 1.15 * t[0], (pair, t)
+
+
 @pytest.mark.parametrize("storage", [0, 1, 2])
 def test_block_size_reaches_small_lattices(gf, storage):
     # every block size is taken, on FP64 storage and on lattices of the direction-per-warp kernel
