@@ -338,9 +338,9 @@ struct gf_handle {
   int phase_sweeps[2] = {0, 0};
   int sweeps_done = 0;  // since the last upload: the reunitarisation / check schedule
   // graphs: per buffer state (OR) one of each length 16, 8, 4, 2, 1 sweeps, one per set
-  // of precision levels of a mixed run, the same lengths for Fourier acceleration
+  // of precision levels of a mixed run and form of its double-float sweep, the same lengths for Fourier acceleration
   cudaGraphExec_t graph[3][5] = {};
-  cudaGraphExec_t graph_mix[8] = {};
+  cudaGraphExec_t graph_mix[16] = {};
   cudaGraphExec_t graph_fasd[6] = {};  // 16, 8, 4, 2, 1 iterations; the measurement after the last
   // pinned host ring: slots 0 and 1 receive the result block (iteration counts, lattice
   // F and theta, loop state) behind each replay in flight, whose events follow the
@@ -862,6 +862,11 @@ int level_storage(const gf_handle* h, int L) { return L == 1 ? h->storage : L ==
 char* level_links(const gf_handle* h, int L) { return L == 1 ? h->links : h->links64; }
 LatDev* level_lats(const gf_handle* h, int L) { return L == 1 ? h->d_lats : h->d_lats64; }
 
+// Whether double-float sweeps of units with this many sites in all take the kernel that stages
+// the links in shared memory (gf_split.cuh, which says where the line lies)
+bool split_staged(long long sites) { return sites * 4 * 144 > (96LL << 20); }
+constexpr int kMixStaged = 8;  // beside the level bits of a mixed graph's key
+
 SweepArgs sweep_args_level(gf_handle* h, int L, int parity, int reverse) {
   SweepArgs a = sweep_args(h, parity, true, reverse);
   a.links = level_links(h, L);
@@ -883,7 +888,7 @@ MeasureArgs measure_args_level(gf_handle* h, int L, int parity, int reverse, boo
   return a;
 }
 
-// One sweep of the mixed loop over the levels in `mask` (bit L-1 for level L): the
+// One sweep of the mixed loop over the levels in `mask` (bit L-1 for level L; kMixStaged): the
 // half-sweeps of every level, then FINISH_ODD; as in the one-level loop, the even-site
 // pass of every level and FINISH_LOOP follow in the graph when there are many units,
 // and an open sweep of one unit is resolved by the host (resolve_open_sweep_levels).
@@ -893,8 +898,9 @@ int enqueue_mixed_sweep(gf_handle* h, cudaStream_t s, int* pass, int mask) {
     rev = (*pass)++ & 1;
     for (int L = 1; L <= 3; ++L)
       if (mask & (1 << (L - 1))) {
-        launch_sweep(level_storage(h, L), h->nd, h->repro, h->variant, sweep_args_level(h, L, parity, rev),
-                     h->n_tiles, h->tile, s);
+        SweepArgs a = sweep_args_level(h, L, parity, rev);
+        a.staged = (mask & kMixStaged) != 0;
+        launch_sweep(level_storage(h, L), h->nd, h->repro, h->variant, a, h->n_tiles, h->tile, s);
         GF_CK_LAUNCH(h);
       }
   }
@@ -996,11 +1002,14 @@ int run_mixed(gf_handle* h, double eps, int budget, int* sweeps_fp32, int* sweep
   *sweeps_fp32 = *sweeps_polish = 0;
   int mask_prev = 0, sweep_prev = 0;
   // tiles per unit, for the compaction of the tile table as units finish
-  std::vector<long long> unit_ntiles(nu, 0);
+  std::vector<long long> unit_ntiles(nu, 0), unit_sites(nu, 0);
   for (int l = 0; l < h->n_lat; ++l) {
     const LatDev& d = h->lats[l];
     const long long per_slice = (d.V3h + h->tile - 1) / h->tile;
-    for (int k = 0; k < d.n_units; ++k) unit_ntiles[d.unit0 + k] = per_slice * (d.L[3] / d.n_units);
+    for (int k = 0; k < d.n_units; ++k) {
+      unit_ntiles[d.unit0 + k] = per_slice * (d.L[3] / d.n_units);
+      unit_sites[d.unit0 + k] = d.V / d.n_units;
+    }
   }
   bool compacted = false;
   // the units of lattice l are lats[l].unit0 .. + n_units - 1
@@ -1051,11 +1060,13 @@ int run_mixed(gf_handle* h, double eps, int budget, int* sweeps_fp32, int* sweep
     if (rc == GF_OK) continue;  // moved units were measured at their new level: read again
     if (s.n_active == 0 || s.sweep >= s.limit) break;
     int mask = 0;
-    long long need = 0;
+    long long need = 0, split_sites = 0;
     for (int u = 0; u < nu; ++u) {
       if (act[u] > 0) mask |= 1 << (act[u] - 1);
+      if (act[u] == 2) split_sites += unit_sites[u];
       if (act[u] != 0) need += unit_ntiles[u];
     }
+    if (split_staged(split_sites)) mask |= kMixStaged;
     if (nu > 1 && 2 * need <= h->n_tiles) {  // half the table or more belongs to finished units
       std::vector<int> keep(nu);
       for (int u = 0; u < nu; ++u) keep[u] = act[u] != 0;

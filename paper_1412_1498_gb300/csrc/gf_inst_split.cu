@@ -13,8 +13,7 @@ cudaError_t prepare_sweep_split() {
 }
 
 void launch_sweep_split(int nd, const SweepArgs& a, int n_tiles, int tile, cudaStream_t s) {
-  const long long link_bytes = 2LL * n_tiles * tile * 4 * 144;  // of the units in the tile table
-  if (link_bytes > (96LL << 20) && tile >= kSplitBlock) {
+  if (a.staged && tile >= kSplitBlock) {
     const size_t smem = (size_t)kSplitWords * kSplitBlock * sizeof(float4);
     if (nd == 4) k_or_sweep_split<4, true><<<n_tiles, kSplitBlock, smem, s>>>(a);
     else k_or_sweep_split<3, true><<<n_tiles, kSplitBlock, smem, s>>>(a);

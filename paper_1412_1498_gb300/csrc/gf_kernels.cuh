@@ -311,6 +311,7 @@ struct SweepArgs {
   int dep;                 // launch with programmatic stream serialisation (launch_dep)
   int dir;                 // the direction-per-warp kernel (small lattices)
   int tile_sites;          // sites a tile covers (fewer at the end of a time slice)
+  int staged;              // double-float sweep: links staged in shared memory (split_staged)
   Relax omega;
 };
 

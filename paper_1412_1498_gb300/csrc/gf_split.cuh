@@ -298,8 +298,10 @@ __device__ __forceinline__ float split_theta_site(const acc2 (&A)[18]) {
 // streaming, which keeps the lines other blocks will reload in L2.  us a sweep, read twice
 // -> staged: 24^4 (191 MB of links) 161 -> 147, 32^4 (604 MB) 453 -> 426, where the second reads
 // that miss L2 cost DRAM a tenth more traffic; 16^4 (38 MB) 36.3 -> 38.8, 20x12x18x10 36.1 -> 41.0,
-// where the larger number of warps counts.  The line is drawn at 96 MB of links in the tile table
-// (L2 holds 126 MB); 96 or 32 sites a block were slower (24^4 192, 179).
+// where the larger number of warps counts.  The line (split_staged) is drawn at 96 MB of links of
+// the units that sweep in double-float (L2 holds 126 MB); a tile table holds units of other
+// levels too, whose blocks would only wait for 74 KB of shared memory to find that out.  96 or 32
+// sites a block were slower (24^4 192, 179).
 constexpr int kSplitBlock = 64;
 constexpr int kSplitWords = 72;  // word w of the side (0 forward, 1 backward) link mu: (2 mu + side) 9 + w
 

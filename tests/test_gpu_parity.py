@@ -706,3 +706,29 @@ def test_block_size_reaches_small_lattices(gf, storage):
     assert storage != gf.GF_FP64_18 or min(ts[256]) > 1.5 * min(ts[128])
     for u, F, th in out[1:]:
         assert np.array_equal(u, out[0][0]) and abs(F - out[0][1]) < 1e-12 and abs(th - out[0][2]) < 1e-12 * th
+
+
+@pytest.mark.parametrize("gauge", [0, 1])
+def test_staged_polish_of_units_that_stop_one_by_one(gf, gauge):
+    # six lattices (6 x 18 MB of links, above the staged sweep's line) that reach the threshold one
+    # after another: the polish goes from the staged kernel to the other one on the way, and
+    # each lattice has the bits and the sweep counts of its run alone, which never took the staged one
+    dims, amps = (16, 12, 10, 16), (0.005, 0.01, 0.015, 0.02, 0.025, 0.03)
+    Us = [fields.smooth_field(dims, a, 97) for a in amps]
+    fx = gf.GaugeFixer([dims] * 6, gauge, gf.GF_FP32_12, mixed=True)
+    gf.gf_set_mixed_switch(fx.h, 1e3)                       # every sweep in double-float
+    for i, U in enumerate(Us):
+        fx.upload(U, i)
+    eps = 1e-9
+    both = fx.fix(eps, 400)
+    n = 1 if gauge == 0 else dims[3]
+    assert len(set(both["iters"].reshape(6, n).max(1).tolist())) > 1
+    for i, U in enumerate(Us):
+        one = gf.GaugeFixer(dims, gauge, gf.GF_FP32_12, mixed=True)
+        gf.gf_set_mixed_switch(one.h, 1e3)
+        one.upload(U)
+        r = one.fix(eps, 400)
+        assert np.array_equal(r["iters"], both["iters"].reshape(6, n)[i])
+        assert np.array_equal(one.download(), fx.download(i))
+        one.close()
+    fx.close()
