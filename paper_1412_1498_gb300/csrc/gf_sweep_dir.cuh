@@ -7,7 +7,8 @@
 // memory; one warp adds the shares, runs the three subgroup steps and leaves g(x) there; each
 // warp then applies g to the two links it still holds.  The warp that does the subgroup
 // steps changes from block to block: warps of one number share a scheduler.
-// The sums run in the order of the one-thread kernels: the same bits.
+// The sums run in the order of the one-thread kernels: the same bits, in the links and in the
+// check's F and theta of a site.
 //
 // us a sweep, one thread a site -> one warp a direction: Landau FP32-12 8^4 12.9 -> 9.9, 8x16x16x8
 // (2^14 sites) 14.0 -> 10.8, 16^3x8 13.9 -> 13.3, 16^4 16.5 -> 20.4; FP32-18 8^4 14.5 -> 10.0,
@@ -42,8 +43,8 @@ __global__ void __launch_bounds__(kDirThreads, dir_min_blocks<S>()) k_or_sweep_d
   using St = Store<S>;
   using T = typename St::T;
   constexpr int NE = St::NE;
-  constexpr bool kCheckGK = sizeof(T) == 4;  // FP64 sums the stored links' A (Eq. (3))
-  __shared__ T ks[4][18][32];                // K shares, later A shares of a check
+  constexpr bool kCheckGK = sizeof(T) == 4;  // FP64 sums the stored links' A - A^dagger (Eq. (3))
+  __shared__ T ks[4][18][32];                // K shares, later Delta shares of a check
   __shared__ T gs[18][32];
   __shared__ T fs4[4][32];
   grid_dep_wait();
@@ -113,12 +114,11 @@ __global__ void __launch_bounds__(kDirThreads, dir_min_blocks<S>()) k_or_sweep_d
       cx<T> fu[9], bu[9];
       to_full(f, fu);
       to_full(b, bu);
+      AntiHermSum<T> D;
+      D.add(fu, bu, true);
+      const T d[9] = {D.d01.re, D.d01.im, D.d02.re, D.d02.im, D.d12.re, D.d12.im, D.e0, D.e1, D.e2};
 #pragma unroll
-      for (int e = 0; e < 9; ++e) {
-        const cx<T> d = csub(bu[e], fu[e]);
-        ks[mu][2 * e][lane] = d.re;
-        ks[mu][2 * e + 1][lane] = d.im;
-      }
+      for (int e = 0; e < 9; ++e) ks[mu][e][lane] = d[e];
       fs4[mu][lane] = (fu[0].re + fu[4].re + fu[8].re) + (bu[0].re + bu[4].re + bu[8].re);
     }
     St::store(base, V, mu, ds.idx_f, f);
@@ -127,17 +127,18 @@ __global__ void __launch_bounds__(kDirThreads, dir_min_blocks<S>()) k_or_sweep_d
   if (!kCheckGK && measure_now) {
     __syncthreads();
     if (mu == turn && valid) {
-      cx<T> A[9];
+      T s[9];
 #pragma unroll
-      for (int e = 0; e < 9; ++e) A[e] = {ks[0][2 * e][lane], ks[0][2 * e + 1][lane]};
+      for (int e = 0; e < 9; ++e) s[e] = ks[0][e][lane];
       fs = fs4[0][lane];
 #pragma unroll
       for (int d = 1; d < ND; ++d) {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) A[e] = cadd(A[e], cx<T>{ks[d][2 * e][lane], ks[d][2 * e + 1][lane]});
+        for (int e = 0; e < 9; ++e) s[e] = s[e] + ks[d][e][lane];
         fs = fs + fs4[d][lane];
       }
-      q = theta_site(A);
+      AntiHermSum<T> D = {{s[0], s[1]}, {s[2], s[3]}, {s[4], s[5]}, s[6], s[7], s[8]};
+      q = D.finish();
     }
   }
   if (measure_now && mu == turn) {

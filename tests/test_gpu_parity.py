@@ -732,3 +732,23 @@ def test_staged_polish_of_units_that_stop_one_by_one(gf, gauge):
         assert np.array_equal(one.download(), fx.download(i))
         one.close()
     fx.close()
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 4), (6, 10, 8, 4), (10, 6, 14, 4)])
+def test_small_fp64_slices_check_as_batch_members(gf, dims, form):
+    # time slices of a small lattice in FP64: the direction-per-warp sweep's check and that of the
+    # kernel for larger handles sum in one order, so F, theta and the stop sweeps are the same bits
+    U, filler = fields.random_gauge_config(dims, 0.4, 95), fields.random_gauge_config((16, 16, 16, 4), 0.4, 96)
+    res = []
+    for lats in ([dims], [dims, (16, 16, 16, 4)]):
+        fx = gf.GaugeFixer(lats, gf.GF_COULOMB, gf.GF_FP64_18)
+        gf.gf_set_overrelax_form(fx.h, form)
+        fx.upload(U, 0)
+        if len(lats) > 1:
+            fx.upload(filler, 1)
+        out = fx.fix(1e-6, 43)
+        res.append((fx.download(0), out["iters"][:dims[3]], out["F"][0], out["theta"][0]))
+        fx.close()
+    (ua, ia, Fa, ta), (ub, ib, Fb, tb) = res
+    assert np.array_equal(ua, ub) and np.array_equal(ia, ib) and Fa == Fb and ta == tb
