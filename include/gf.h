@@ -292,6 +292,12 @@ GF_API int gf_set_polish(gf_handle *h, int polish);
 #define GF_SWEEP_PIPELINED 2
 GF_API int gf_set_sweep_variant(gf_handle *h, int variant);
 
+/* Most polls of one wait of the cooperative loop's blocks for each other [2^21, a second or
+   more].  A wait that runs out ends the loop and gf_fix returns GF_ECUDA, with the field
+   somewhere in the sweep: upload it again.  0: every wait runs out (to test a caller's
+   handling of the error). */
+GF_API int gf_set_loop_wait(gf_handle *h, int polls);
+
 /* Autotuner: times 7 sweeps (2 warm-up) of the current field for each block size (64,
    128, 256) and sweep kernel (register / pipelined for FP32-12) with CUDA events on the
    handle's stream and keeps the fastest; *threads_out, *variant_out (nullable) receive

@@ -321,6 +321,7 @@ struct gf_handle {
   Relax relax = relax_of(1.7);  // omega as the kernels take it
   int form = GF_OR_FIRST_ORDER, reunit_interval = 20, check_interval = 1;
   int variant = GF_SWEEP_AUTO;
+  unsigned loop_polls = 1u << 21;  // a second or more
   int polish = GF_POLISH_SPLIT;
   int method = GF_METHOD_OR;
   double alpha = 0.08;
@@ -822,6 +823,7 @@ int run_phase_loop(gf_handle* h, double eps, int budget, int* done) {
   a.n_units = h->n_units;
   a.n_lat = h->n_lat;
   a.nd = h->nd;
+  a.polls = h->loop_polls;
   a.omega = h->relax;
   for (int before = offset - 1;;) {
     const cudaError_t e = launch_loop(h->storage, h->nd, a, h->stream);
@@ -1743,6 +1745,13 @@ int gf_set_polish(gf_handle* h, int polish) {
   if (!h) return GF_EINVAL;
   if (polish != GF_POLISH_FP64 && polish != GF_POLISH_SPLIT) return fail(h, GF_EINVAL, "unknown polish mode");
   h->polish = polish;
+  return GF_OK;
+}
+
+int gf_set_loop_wait(gf_handle* h, int polls) {
+  if (!h) return GF_EINVAL;
+  if (polls < 0) return fail(h, GF_EINVAL, "polls must be >= 0");
+  h->loop_polls = (unsigned)polls;
   return GF_OK;
 }
 

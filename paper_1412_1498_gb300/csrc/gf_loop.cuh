@@ -8,8 +8,8 @@
 // kLoopSweeps sweeps.
 //
 // The kernel is launched cooperatively, so all blocks are resident and the barrier ends.  Its
-// wait is bounded all the same: a block that gives up sets DevState.fault and leaves, the
-// others follow, and the host reports an error.
+// wait is bounded all the same (LoopArgs.polls): a block that gives up sets DevState.fault and
+// leaves, the others follow, and the host reports an error.
 //
 // A sweep: even half-sweep | odd half-sweep, with F and the odd-site theta per tile | the
 // totals of each unit by one block and the decisions of FINISH_ODD | where some unit is
@@ -58,26 +58,27 @@ struct LoopArgs {
   double* lat_theta;
   DevState* st;
   int n_tiles, n_units, n_lat, nd;
+  unsigned polls;          // most polls of one barrier wait
   Relax omega;
 };
 
 // Barrier over the grid: `target` arrivals since the launch (a multiple of the grid size).
 // false: some block gave up.
-__device__ __forceinline__ bool loop_barrier(DevState* st, unsigned target, int* s_ok) {
+__device__ __forceinline__ bool loop_barrier(DevState* st, unsigned target, unsigned polls, int* s_ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(&st->arrived, 1u);
     int ok = 1;
     for (unsigned spins = 0;; ++spins) {
-      unsigned n;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(n) : "l"(&st->arrived) : "memory");
-      if (n >= target) break;
-      if (spins > (1u << 21)) {  // a second or more
+      if (spins >= polls) {
         atomicExch(&st->fault, 1);
         ok = 0;
         break;
       }
+      unsigned n;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(n) : "l"(&st->arrived) : "memory");
+      if (n >= target) break;
     }
     __threadfence();
     *s_ok = ok && *(volatile int*)&st->fault == 0;
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kLoopThreads, 2) k_loop(LoopArgs a) {
 #define BARRIER()                                             \
   do {                                                        \
     target += (unsigned)G;                                    \
-    if (!loop_barrier(a.st, target, &s_ok)) return;           \
+    if (!loop_barrier(a.st, target, a.polls, &s_ok)) return;           \
   } while (0)
   while (n_active > 0 && sweep < limit && sweep - sweep0 < kLoopSweeps) {
     const bool check = ((sweep + 1) % ci) == 0 || sweep + 1 == limit;

@@ -66,6 +66,7 @@ _SIGS = {
     "gf_set_block_size": (_int, [_vp, _int]),
     "gf_fix_phase_sweeps": (_int, [_vp, _IP, _IP]),
     "gf_set_sweep_variant": (_int, [_vp, _int]),
+    "gf_set_loop_wait": (_int, [_vp, _int]),
     "gf_set_polish": (_int, [_vp, _int]),
     "gf_autotune": (_int, [_vp, _IP, _IP]),
     "gf_get_sweeps_done": (_int, [_vp, _IP]),
@@ -239,6 +240,10 @@ def gf_set_polish(h, polish: int) -> None:
 
 def gf_set_sweep_variant(h, variant: int) -> None:
     _check(_lib.gf_set_sweep_variant(h, variant), h)
+
+
+def gf_set_loop_wait(h, polls: int) -> None:
+    _check(_lib.gf_set_loop_wait(h, polls), h)
 
 
 def gf_autotune(h):

@@ -752,3 +752,43 @@ def test_small_fp64_slices_check_as_batch_members(gf, dims, form):
         fx.close()
     (ua, ia, Fa, ta), (ub, ib, Fb, tb) = res
     assert np.array_equal(ua, ub) and np.array_equal(ia, ib) and Fa == Fb and ta == tb
+
+
+def test_loop_wait_that_runs_out_is_an_error(gf):
+    # no poll allowed: every block gives up at the first barrier and leaves; the handle goes on
+    dims = (6, 10, 8, 4)
+    U = fields.random_gauge_config(dims, 0.4, 93)
+    fx = gf.GaugeFixer(dims, gf.GF_COULOMB, gf.GF_FP32_12)
+    fx.upload(U)
+    good = fx.fix(1e-300, 12), fx.download()
+    gf.gf_set_loop_wait(fx.h, 0)
+    fx.upload(U)
+    with pytest.raises(gf.GFError) as e:
+        fx.fix(1e-300, 12)
+    assert e.value.code == gf.GF_ECUDA and "waiting" in str(e.value)
+    gf.gf_set_loop_wait(fx.h, 1 << 21)
+    fx.upload(U)
+    again = fx.fix(1e-300, 12)
+    assert np.array_equal(fx.download(), good[1]) and again["theta"][0] == good[0]["theta"][0]
+    with pytest.raises(gf.GFError):
+        gf.gf_set_loop_wait(fx.h, -1)
+    fx.close()
+
+
+@pytest.mark.parametrize("storage", [1, 2])
+def test_small_handle_loop_continues_over_launches(gf, storage):
+    # a launch serves 4096 sweeps at most: 9001 take three, with the schedules carried over; the
+    # launched loop (block size 64) gives the same links, counts and, to the order of the sums, values
+    dims = (4, 4, 6, 2)
+    U = fields.random_gauge_config(dims, 0.4, 92)
+    res = []
+    for threads in (128, 64):
+        fx = gf.GaugeFixer(dims, gf.GF_COULOMB, storage)
+        gf.gf_set_block_size(fx.h, threads)
+        gf.gf_set_check_interval(fx.h, 7)
+        fx.upload(U)
+        r = fx.fix(1e-300, 9001)
+        res.append((fx.download(), r["iters"], gf.gf_get_sweeps_done(fx.h), r["F"][0]))
+        fx.close()
+    assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
+    assert res[0][2] == res[1][2] == 9001 and abs(res[0][3] - res[1][3]) < 1e-12
