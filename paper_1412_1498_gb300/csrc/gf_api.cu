@@ -1487,6 +1487,17 @@ const double* host_mapped(const double* p) {
   return static_cast<const double*>(at.devicePointer);
 }
 
+// Whether a pointer given as device memory is memory of a device.  Pinned host and managed memory are
+// as usable for loads and stores of a kernel, but a bulk copy is not asked to write there.
+static bool is_device_memory(const double* p) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice;
+}
+
 int gf_upload(gf_handle* h, int lat, const double* links, int on_device) {
   if (!h) return GF_EINVAL;
   if (lat < 0 || lat >= h->n_lat || !links) return fail(h, GF_EINVAL, "bad lattice index or null buffer");
@@ -1522,7 +1533,8 @@ int gf_download(gf_handle* h, int lat, double* links, int on_device) {
   const int st = cur_storage(h);
   double* mapped = on_device ? nullptr : const_cast<double*>(host_mapped(links));
   if (on_device || mapped) {
-    launch_unpack(st, cur_links(h), d, on_device ? links : mapped, 0, d.V, on_device != 0, h->stream);
+    launch_unpack(st, cur_links(h), d, on_device ? links : mapped, 0, d.V, on_device && is_device_memory(links),
+                  h->stream);
     GF_CK_LAUNCH(h);
     if (mapped) GF_CK(h, cudaStreamSynchronize(h->stream));
   } else {

@@ -251,3 +251,26 @@ def test_conversion_is_the_cast(gf, storage, special):
             got = got if isinstance(got, np.ndarray) else got.cpu().numpy()
             assert np.array_equal(got[..., :rows, :].view(np.uint64), want[..., :rows, :].copy().view(np.uint64))
     fx.close()
+
+
+def test_download_without_a_synchronise(gf):
+    # on_device = 1 with device memory, also inside a stream capture, and with pinned host memory
+    # (which a kernel can write as well): asynchronous on the stream, the same links
+    dims = (4, 6, 4, 2)
+    U = torch.from_numpy(fields.random_gauge_config(dims, 0.5, 12)).cuda()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        fx = gf.GaugeFixer(dims, gf.GF_LANDAU, gf.GF_FP32_12)
+        fx.upload(U)
+        want, got = torch.empty_like(U), torch.empty_like(U)
+        fx.download(0, want)
+        pinned = torch.empty(U.shape, dtype=U.dtype, pin_memory=True)
+        gf.gf_download(fx.h, 0, pinned.data_ptr(), True)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            fx.download(0, got)
+        graph.replay()
+        s.synchronize()
+        fx.close()
+    assert torch.equal(pinned, want.cpu()) and torch.equal(got, want)
