@@ -272,7 +272,9 @@ GF_API int gf_set_block_size(gf_handle *h, int threads);      /* [128]; 64, 128 
      2^14 sites in all: a warp per direction;
    - FP64 storages above that: blocks of one warp;
    - gf_fix of several units on up to 2^17 sites in FP32-12 or FP32-18 (first-order form, no
-     history, at most 128 units, not mixed): the loop in one cooperative kernel.
+     history, at most 128 units, not mixed): the loop in one cooperative kernel.  Several
+     such handles at work on streams of their own share the GPU better with a block size of
+     64, or as one batch.
    The links are the same bits with every choice. */
 /* Arithmetic of the polish phase of a mixed-precision gf_fix (GF_FLAG_MIXED):
    GF_POLISH_SPLIT [default]: double-float sweeps (each real an unevaluated sum of two

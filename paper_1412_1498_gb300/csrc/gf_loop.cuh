@@ -21,11 +21,16 @@
 // overrelaxation runs here: nvcc contracts the exact form's products otherwise than in the
 // sweep kernels, and the links would not be the same bits.
 //
-// Coulomb gauge FP32-12, us a sweep, launches -> this kernel: 8^3x16 21.2 -> 14.8, 12^3x16
-// 21.8 -> 15.2, 16^3x32 32.4 -> 26.1 (above that the pipelined kernels' bandwidth counts for
-// more).  A one-unit handle has three launches a sweep and gained nothing (8^4 12.2 against 12.7,
+// Coulomb gauge, us a sweep, launches (blocks of 64 sites) -> this kernel: FP32-12 8^3x16 22.7 -> 14.8,
+// 12^3x16 22.9 -> 15.5, 16^4 24.4 -> 17.9, 16^3x32 33.5 -> 26.0 (above that the pipelined kernels'
+// bandwidth counts for more); FP32-18 23.5 -> 16.8, 23.6 -> 18.1, 26.7 -> 20.0, 38.9 -> 30.4.  A
+// one-unit handle has three launches a sweep and gained nothing (8^4 12.2 against 12.7,
 // 16^4 16.9 against 16.9), nor did a warp per direction here (8^4 11.5, 16^4 23.1): it keeps its
-// launches.
+// launches.  Loops of several handles on streams of their own run side by side as far as their
+// blocks fit the GPU together, and one after another beyond that, where launched loops share it: us a
+// sweep over 1, 2, 4, 8 handles together, launches -> this kernel, 8^3x16 23.6 14.0 7.1 4.5 -> 15.6
+// 8.5 4.6 3.6; 12^3x16 24.5 13.3 7.3 5.1 -> 15.6 8.5 8.5 8.6; 16^3x32 36.1 23.1 19.7 21.0 -> 26.2 25.7
+// 26.0 26.0.  Such callers batch the lattices in one handle or take a block size of 64.
 #pragma once
 
 #include "gf_kernels.cuh"

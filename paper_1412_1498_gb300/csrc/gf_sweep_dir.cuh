@@ -11,10 +11,10 @@
 // check's F and theta of a site.
 //
 // us a sweep, one thread a site -> one warp a direction: Landau FP32-12 8^4 12.9 -> 9.9, 8x16x16x8
-// (2^14 sites) 14.0 -> 10.8, 16^3x8 13.9 -> 13.3, 16^4 16.5 -> 20.4; FP32-18 8^4 14.5 -> 10.0,
-// 2^14 sites 14.5 -> 11.4; FP64-18 8^4 94.8 -> 49.9, 2^14 sites 95.7 -> 77.1, 16^3x8 105 -> 130.  So
-// the line is 2^14 sites.  Above it the SMs are full enough, and the barriers between the
-// phases cost more than they give (24^4 FP32-18, 20 sweeps: 1.49 -> 1.64 ms).
+// (2^14 sites) 13.8 -> 11.2, 16^3x8 15.4 -> 14.0, 16^4 16.9 -> 21.9; FP32-18 8^4 14.0 -> 10.6,
+// 2^14 sites 16.6 -> 11.8, 16^3x8 17.4 -> 15.4, 16^4 19.0 -> 23.8; FP64-18 8^4 94.8 -> 46.6, 2^14 sites
+// 95.5 -> 73.4, 16^3x8 101 -> 115.  So the line is 2^14 sites.  Above it the SMs are full enough, and
+// the barriers between the phases cost more than they give (24^4 FP32-18 66.7 -> 78.7).
 #pragma once
 
 #include "gf_kernels.cuh"
