@@ -304,9 +304,9 @@ GF_API int gf_set_loop_wait(gf_handle *h, int polls);
    128, 256) and sweep kernel (register / pipelined for FP32-12) with CUDA events on the
    handle's stream and keeps the fastest; *threads_out, *variant_out (nullable) receive
    the choice, and setting them on another handle of the same lattices makes the same one.
-   Handles that gf_fix serves with one cooperative kernel keep the defaults.  The timing sweeps are applied to the field (they are gauge
-   transformations of it): tune before uploading the field to fix, or upload it again
-   afterwards.  Synchronises the stream. */
+   Handles that gf_fix serves with one cooperative kernel keep the defaults.  The timing
+   sweeps are applied to the field (they are gauge transformations of it): tune before
+   uploading the field to fix, or upload it again afterwards.  Synchronises the stream. */
 GF_API int gf_autotune(gf_handle *h, int *threads_out, int *variant_out);
 
 /* Checkpoint / resume.  The handle counts the sweeps (or Fourier-accelerated iterations)

@@ -1782,7 +1782,7 @@ int gf_set_sweep_variant(gf_handle* h, int variant) {
 
 // One sweep as the tuner times it: as gf_fix's loop runs it, with the check of a check sweep in
 // the odd half-sweep (without it the register kernel looks as fast as the pipelined one and is a
-// tenth slower in the loop: Coulomb 32^3x64 0.299 against 0.255 ms a sweep).
+// tenth and more slower in the loop: Coulomb 32^3x64 0.312 against 0.271 ms a sweep).
 static int tuning_sweep(gf_handle* h) {
   const int st = cur_storage(h);
   for (int p = 0; p < 2; ++p) {
